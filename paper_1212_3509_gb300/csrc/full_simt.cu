@@ -2,101 +2,298 @@
 //
 // Cor. 3 (Eq. kron_operator) with the mode product of Sec. 2.2 (Eq. modemul):
 // per node k and component q the three Toeplitz factors act along i1, i2, i3.
-// Per node the nine products share work (8 GEMMs of n^4 multiply-adds):
-//   mode 1:  Y1 = m1 x_1 F,  Y2 = m2 x_1 E,  Y3 = m3 x_1 E
-//   mode 2:  U = Y1 x_2 E + Y2 x_2 F,  V = Y3 x_2 E
-//   mode 3:  phi = sum_k (U_k x_3 S_k E + V_k x_3 S_k F),  S_k = c s omega_k
-// and the node sum of the last stage is one contraction of length 2 n3 M.
+// The modes are applied in the order 3, 2, 1.  Per node the nine products
+// share work (8 products of n^4 multiply-adds):
+//   axis 3:  Y_q = m_q x_3 S_k E (q = 1, 2),  Y_3 = m_3 x_3 S_k F,  S_k = c s omega_k
+//   axis 2:  U = Y_2 x_2 F + Y_3 x_2 E,  V = Y_1 x_2 E
+//   axis 1:  phi = sum_k (U_k x_1 E + V_k x_1 F)
+// and the node sum of the last stage is one contraction of length 2 n1 M.
+// Every field stays in the caller's layout [i3][i2][i1]: along axes 3 and 2
+// the rows of a product (everything but the contracted index) are contiguous
+// or in contiguous runs of n1, so nothing is ever transposed; only the last
+// stage reads its contraction index contiguously.
 //
-// Every stage is a "TN" GEMM whose output is stored transposed:
-//   C[a][row] = alpha * sum_pairs sum_kk A[row][kk] * B[a][kk],
-// A = the field with its contraction index contiguous, B = the n x n factor.
-// Storing [a][row] rotates the axes (i3,i2,i1) -> (i1,i3,i2) -> (i2,i1,i3) ->
-// (i3,i2,i1), so every stage reads its contraction index contiguously and the
-// final stage writes phi in [i3][i2][i1] order.  The same kernel serves the
-// adjoint (one field in, three out) and the FP64 form.
-#include <vector>
+// Even / odd halves.  With x+_j = x_j + x_{n-1-j} and x-_j = x_j - x_{n-1-j}
+// (j < h = ceil(n/2)) a symmetric Toeplitz factor maps x+ to the even half
+// p_a = (y_a + y_{n-1-a})/2 of the output and x- to the odd half
+// q_a = (y_a - y_{n-1-a})/2, a skew one the other way round, so a product
+// takes half the multiply-adds of the dense factor.  The sums x+- are formed
+// while a tile is loaded and y_a = p_a + q_a, y_{n-1-a} = p_a - q_a in its
+// epilogue: no folded copy of any field exists.  A factor without that
+// symmetry (non-uniform grid) is the sum of two such parts.
+#include <climits>
+#include <cmath>
+#include <cooperative_groups.h>
+#include <mutex>
+#include <type_traits>
 
 #include "internal.h"
 
 namespace demag {
 
-constexpr int kMaxJobs = 64;
-constexpr int kMaxPairs = 3 * kMaxTerms + 8;  // the adjoint node sum: 3 jobs of M pairs
+constexpr int kMaxPairs = 4;  // (field, factor part) pairs summed by one output field of one node
 
-struct GemmJob {
-  int rows, ncol, K;
-  int lda, ldb, ldc;
-  int pair0, npairs;
-  int tiles_m, tiles_n, tile0;
-  float alpha;
-  void* C;
+// One launch: outputs (node, job), each sum over its pairs of a half-matrix
+// product along one axis.  Element (row r, index j) of a field is at
+// (r / inner) * ostride + r % inner + j * kstride.
+struct ModeStage {
+  int n, h, ldh;          // contracted axis, ceil(n / 2), leading dimension of the factor parts
+  int inner;              // contiguous rows
+  unsigned inner_mul, inner_shift;  // r / inner = (umulhi(r, inner_mul) + r) >> inner_shift
+  long ostride, kstride;
+  int rows;               // rows of one field
+  long N;                 // elements of one field
+  const void* A;          // input fields
+  const void* B;          // factor parts of this axis, first node of the launch
+  void* C;                // output fields
+  long b_node;            // elements between the factor parts of consecutive nodes
+  int nodes;              // nodes of this launch: one output per node, or summed (SUM)
+  int a_node, c_node;     // fields per node in A (0: shared by the nodes) and C
+  int njobs;              // outputs per node
+  int npairs[3];          // pairs per output
+  int a_field[3][kMaxPairs];
+  long b_off[3][kMaxPairs];
+  int swap[3][kMaxPairs]; // 0: even half from x+, odd from x-; 1: the other way round
+  int tiles_n;
+  int split;              // SUM: node ranges, one per block of a cluster
+  float alpha;            // SUM: scale of the result
 };
 
-struct GemmBatch {
-  int njobs, total_tiles;
-  GemmJob jobs[kMaxJobs];
-  const void* A[kMaxPairs];
-  const void* B[kMaxPairs];
+// ---------------------------------------------------------------- the kernel
+//
+// Bound: the FP32 (FP64) pipe, and close behind it the words that shared
+// memory delivers to registers (32 per cycle and SM against 128 multiply-adds).
+// A block owns BM rows x BN columns of both output halves, a thread TM x TN of
+// each.  The two halves travel as pairs: (x+, x-) of a row and (even, odd) of a
+// factor entry are neighbours in shared memory and one packed operand of
+// fma.rn.f32x2, whose result is the pair of accumulators (the roundings of two
+// fmaf).  2 (TM + TN) words then feed 2 TM TN multiply-adds: with 8 x 8 both
+// pipes are equally full, which is why the widest tile has 128 accumulators.
+// Factor parts go to shared memory by cp.async in their global layout; x+- are
+// formed from registers loaded while the previous operands are used.
+constexpr int kBK = 8;
+
+template <typename T, int BM_, int BN_, int TM_, int TN_, int OCC_>
+struct ModeCfg {
+  static constexpr int OCC = OCC_;                 // resident blocks the registers are bounded for
+  static constexpr int BM = BM_, BN = BN_, TM = TM_, TN = TN_;
+  static constexpr int WR = BM / (8 * TM), WC = BN / (4 * TN);  // warps along rows and columns, 8 x 4 threads each
+  static constexpr int NT = 32 * WR * WC;
+  static constexpr int VA = 8 / (int)sizeof(T);    // pairs per 16-byte read
+  static constexpr int LDA = BM + 2;               // 16-byte rows; the offset spreads transposed stores over the banks
+  static constexpr int LA = BM * kBK / NT;
+  static constexpr int LB = BN * kBK / VA;         // 16-byte copies of a factor block
+  static constexpr size_t operands = (size_t)2 * kBK * (LDA + BN) * 2 * sizeof(T);
+  static constexpr size_t reduce = (size_t)2 * BM * BN * sizeof(T);
+  static_assert(LA * NT == BM * kBK && WR * 8 * TM == BM && WC * 4 * TN == BN, "tiles divide evenly");
 };
 
-template <typename T> struct SimtCfg;
-template <> struct SimtCfg<float> { static constexpr int TM = 8, BK = 8; };
-template <> struct SimtCfg<double> { static constexpr int TM = 4, BK = 8; };
+// r / inner and r % inner by multiplication (rows stay below 2^31)
+template <int KIND>
+__device__ __forceinline__ long row_offset(const ModeStage& S, int r) {
+  if (KIND == 0) return r;  // axis 3: all rows are one run
+  if (KIND == 2) return r * S.ostride;
+  const int q = (int)((__umulhi((unsigned)r, S.inner_mul) + (unsigned)r) >> S.inner_shift);
+  return q * S.ostride + (r - q * S.inner);
+}
 
-// 256 threads as 16 x 16; each thread owns TM rows x TM columns of the tile.
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_tn_kernel(const __grid_constant__ GemmBatch batch) {
-  constexpr int TM = SimtCfg<T>::TM, BK = SimtCfg<T>::BK;
-  constexpr int BM = 16 * TM, BN = 16 * TM;
-  constexpr int LA = BM * BK / 256;  // elements each thread loads per operand
-  __shared__ T As[2][BK][BM + 4];  // +4: conflict-free transposed stores
-  __shared__ T Bs[2][BK][BN + 4];
+__device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
 
-  int tile = blockIdx.x;
-  int j = 0;
-  while (j + 1 < batch.njobs && tile >= batch.jobs[j + 1].tile0) ++j;
-  const GemmJob& J = batch.jobs[j];
-  tile -= J.tile0;
-  const int tm = tile % J.tiles_m, tn = tile / J.tiles_m;
-  const int row0 = tm * BM, col0 = tn * BN;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-
-  T acc[TM][TM];
+// A thread's accumulators of both halves: TM x TN pairs.
+template <typename Cfg, typename T> struct ModeAcc;
+template <typename Cfg> struct ModeAcc<Cfg, float> {
+  unsigned long long v[Cfg::TM][Cfg::TN];
+  __device__ __forceinline__ void clear() {
 #pragma unroll
-  for (int a = 0; a < TM; ++a)
+    for (int i = 0; i < Cfg::TM; ++i)
 #pragma unroll
-    for (int b = 0; b < TM; ++b) acc[a][b] = (T)0;
-
-  const int nk = (J.K + BK - 1) / BK;
-  const int steps = nk * J.npairs;
-  T ra[LA], rb[LA];
-
-  auto load = [&](int step) {
-    const int pr = J.pair0 + step / nk;
-    const int k0 = (step % nk) * BK;
-    const T* A = (const T*)batch.A[pr];
-    const T* B = (const T*)batch.B[pr];
+      for (int j = 0; j < Cfg::TN; ++j) v[i][j] = 0ull;
+  }
+  __device__ __forceinline__ float get(int s, int i, int j) const {
+    return __uint_as_float((unsigned)(s ? v[i][j] >> 32 : v[i][j] & 0xffffffffull));
+  }
+  // += pairs of rows (at ax) * pairs of factor entries (at bx)
+  __device__ __forceinline__ void step(const float2* ax, const float2* bx) {
+    unsigned long long a[Cfg::TM], b[Cfg::TN];
 #pragma unroll
-    for (int i = 0; i < LA; ++i) {
-      int idx = threadIdx.x + i * 256;
-      int r = idx / BK, kk = idx % BK;
-      int gk = k0 + kk;
-      int gr = row0 + r, gc = col0 + r;
-      ra[i] = (gr < J.rows && gk < J.K) ? A[(long)gr * J.lda + gk] : (T)0;
-      rb[i] = (gc < J.ncol && gk < J.K) ? B[(long)gc * J.ldb + gk] : (T)0;
+    for (int c = 0; c < Cfg::TM / 2; ++c) {
+      const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(ax + c * 16);
+      a[2 * c] = u.x;
+      a[2 * c + 1] = u.y;
+    }
+#pragma unroll
+    for (int j = 0; j < Cfg::TN / 2; ++j) {
+      const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(bx + 2 * j);
+      b[2 * j] = u.x;
+      b[2 * j + 1] = u.y;
+    }
+#pragma unroll
+    for (int i = 0; i < Cfg::TM; ++i)
+#pragma unroll
+      for (int j = 0; j < Cfg::TN; ++j) fma2(v[i][j], a[i], b[j]);
+  }
+};
+template <typename Cfg> struct ModeAcc<Cfg, double> {
+  double v[2][Cfg::TM][Cfg::TN];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int i = 0; i < Cfg::TM; ++i)
+#pragma unroll
+        for (int j = 0; j < Cfg::TN; ++j) v[s][i][j] = 0.0;
+  }
+  __device__ __forceinline__ double get(int s, int i, int j) const { return v[s][i][j]; }
+  __device__ __forceinline__ void step(const double2* ax, const double2* bx) {
+    double2 a[Cfg::TM], b[Cfg::TN];
+#pragma unroll
+    for (int i = 0; i < Cfg::TM; ++i) a[i] = ax[i * 8];
+#pragma unroll
+    for (int j = 0; j < Cfg::TN; ++j) b[j] = bx[j];
+#pragma unroll
+    for (int i = 0; i < Cfg::TM; ++i)
+#pragma unroll
+      for (int j = 0; j < Cfg::TN; ++j) {
+        v[0][i][j] = fma(a[i].x, b[j].x, v[0][i][j]);
+        v[1][i][j] = fma(a[i].y, b[j].y, v[1][i][j]);
+      }
+  }
+};
+
+template <typename T> struct Pair;
+template <> struct Pair<float> { using type = float2; };
+template <> struct Pair<double> { using type = double2; };
+
+// 16 bytes to shared memory, zeros instead when !ok
+__device__ __forceinline__ void copy16(void* dst, const void* src, bool ok) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+
+// KIND 0: axis 3 (reads the caller's FP32 fields), 1: axis 2, 2: axis 1 with the node sum (contraction
+// index contiguous; writes the caller's FP32 fields; the node ranges of a cluster's blocks are added in
+// rank order through distributed shared memory)
+template <typename T, typename Cfg, int KIND>
+__global__ void __launch_bounds__(Cfg::NT, Cfg::OCC) mode_kernel(const __grid_constant__ ModeStage S) {
+  constexpr bool SUM = KIND == 2, KCONTIG = KIND == 2;
+  using TA = typename std::conditional<KIND == 0, float, T>::type;
+  using TC = typename std::conditional<KIND == 2, float, T>::type;
+  using P2 = typename Pair<T>::type;
+  constexpr int BM = Cfg::BM, BN = Cfg::BN, NT = Cfg::NT, LA = Cfg::LA, LB = Cfg::LB, LDA = Cfg::LDA;
+  constexpr int TM = Cfg::TM, TN = Cfg::TN, VA = Cfg::VA;
+  extern __shared__ __align__(16) unsigned char mode_smem[];
+  P2* const As = reinterpret_cast<P2*>(mode_smem);  // [2 buffers][BK][LDA]: (x+, x-), or (x-, x+) for a swapped pair
+  P2* const Bs = As + 2 * kBK * LDA;                // [2 buffers][BK][BN]: (to the even, to the odd output half)
+
+  const int tid = threadIdx.x;
+  const int rank = SUM ? (int)(blockIdx.x % S.split) : 0;
+  int tile = SUM ? blockIdx.x / S.split : blockIdx.x;
+  const int tn = tile % S.tiles_n;
+  tile /= S.tiles_n;
+  const int job = tile % S.njobs;
+  tile /= S.njobs;
+  int k0 = 0, k1 = 1;
+  if (SUM) {
+    k0 = S.nodes * rank / S.split;
+    k1 = S.nodes * (rank + 1) / S.split;
+  } else {
+    k0 = tile % S.nodes;
+    tile /= S.nodes;
+    k1 = k0 + 1;
+  }
+  const int row0 = tile * BM;
+  const int col0 = tn * BN;
+  const int npairs = S.npairs[job];
+  const int nkb = (S.h + kBK - 1) / kBK;
+  const int steps = (k1 - k0) * npairs * nkb;
+
+  // The elements (index lk(i), row lr(i)) this thread loads per step: consecutive threads on consecutive
+  // rows or, with the contraction index contiguous, on 8 indices of one row.
+  constexpr int RP = KCONTIG ? LA : (BM > NT ? BM / NT : 1);  // different rows
+  constexpr int KSTEP = BM > NT ? 1 : NT / BM;
+  static_assert(KCONTIG || (BM > NT ? BM % NT == 0 : NT % BM == 0), "row mapping");
+  auto lk = [&](int i) { return KCONTIG ? tid % kBK : (BM > NT ? i / RP : tid / BM + i * KSTEP); };
+  auto lr = [&](int i) { return KCONTIG ? tid / kBK + i * (NT / kBK) : (BM > NT ? tid + (i % RP) * NT : tid % BM); };
+  long rbase[RP];
+  bool rok[RP];
+#pragma unroll
+  for (int i = 0; i < RP; ++i) {
+    const int r = row0 + lr(i);
+    rok[i] = r < S.rows;
+    rbase[i] = row_offset<KIND>(S, r);
+  }
+
+  // raw entries x_j, x_{n-1-j} of the next operands: their sums are formed when they are stored, so
+  // that no arithmetic waits for the loads while the current operands are used
+  TA ax[LA], ay[LA];
+  int ld_sw = 0;
+  int ld_k = k0, ld_p = 0, ld_kb = 0;  // what the next load fetches
+  auto load = [&](int buf) {
+    const TA* A = reinterpret_cast<const TA*>(S.A) + ((long)ld_k * S.a_node + S.a_field[job][ld_p]) * S.N;
+    const P2* B = reinterpret_cast<const P2*>(reinterpret_cast<const T*>(S.B) + (long)ld_k * S.b_node +
+                                              S.b_off[job][ld_p]);
+    ld_sw = S.swap[job][ld_p];
+    const int j0 = ld_kb * kBK;
+    const bool whole = j0 + kBK <= S.h;
+    P2* b = Bs + buf * kBK * BN;
+#pragma unroll
+    for (int i = 0; i < (LB + NT - 1) / NT; ++i) {
+      const int e = tid + i * NT, kk = e / (BN / VA), a = e % (BN / VA) * VA;
+      if (LB % NT == 0 || e < LB) {
+        const bool ok = (whole || j0 + kk < S.h) && col0 + a < S.ldh;
+        copy16(b + kk * BN + a, ok ? B + (j0 + kk) * S.ldh + col0 + a : B, ok);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (whole && row0 + BM <= S.rows) {  // no bounds: addresses advance by fixed strides
+      const long d = KCONTIG ? (NT / kBK) * S.ostride : KSTEP * S.kstride;
+      const long ox = (j0 + lk(0)) * S.kstride, oy = (S.n - 1 - j0 - lk(0)) * S.kstride;
+#pragma unroll
+      for (int i = 0; i < LA; ++i) {
+        const TA* p = A + rbase[KCONTIG ? 0 : i % RP];
+        const int t = KCONTIG ? i : i / RP;
+        ax[i] = p[ox + t * d];
+        ay[i] = p[KCONTIG ? oy + t * d : oy - t * d];
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < LA; ++i) {
+        const int ri = i % RP, j = j0 + lk(i);
+        ax[i] = ay[i] = (TA)0;
+        if (rok[ri] && j < S.h) {
+          ax[i] = A[rbase[ri] + j * S.kstride];
+          ay[i] = A[rbase[ri] + (S.n - 1 - j) * S.kstride];
+        }
+      }
+    }
+    if (++ld_kb == nkb) {
+      ld_kb = 0;
+      if (++ld_p == npairs) {
+        ld_p = 0;
+        ++ld_k;
+      }
     }
   };
   auto store = [&](int buf) {
+    P2* a = As + buf * kBK * LDA;
 #pragma unroll
     for (int i = 0; i < LA; ++i) {
-      int idx = threadIdx.x + i * 256;
-      int r = idx / BK, kk = idx % BK;
-      As[buf][kk][r] = ra[i];
-      Bs[buf][kk][r] = rb[i];
+      const T x = (T)ax[i], y = (T)ay[i];
+      P2 v;
+      v.x = ld_sw ? x - y : x + y;
+      v.y = ld_sw ? x + y : x - y;
+      a[lk(i) * LDA + lr(i)] = v;
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
   };
 
+  const int warp = tid / 32, lane = tid % 32;
+  const int wr = (warp % Cfg::WR) * (8 * TM) + (lane % 8) * VA;  // row of accumulator i: wr + (i / VA) 8 VA + i % VA
+  const int wc = (warp / Cfg::WR) * (4 * TN) + (lane / 8) * TN;  // column of accumulator j: wc + j
+  ModeAcc<Cfg, T> acc;
+  acc.clear();
   if (steps > 0) {
     load(0);
     store(0);
@@ -104,176 +301,385 @@ __global__ void __launch_bounds__(256) gemm_tn_kernel(const __grid_constant__ Ge
   __syncthreads();
   for (int s = 0; s < steps; ++s) {
     const int cur = s & 1;
-    if (s + 1 < steps) load(s + 1);
+    if (s + 1 < steps) load(cur ^ 1);
+    const P2* a = As + cur * kBK * LDA + wr;
+    const P2* b = Bs + cur * kBK * BN + wc;
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T av[TM], bv[TM];
-#pragma unroll
-      for (int a = 0; a < TM / 2; ++a) {
-        av[a] = As[cur][kk][tx * (TM / 2) + a];
-        av[a + TM / 2] = As[cur][kk][BM / 2 + tx * (TM / 2) + a];
-        bv[a] = Bs[cur][kk][ty * (TM / 2) + a];
-        bv[a + TM / 2] = Bs[cur][kk][BN / 2 + ty * (TM / 2) + a];
-      }
-#pragma unroll
-      for (int a = 0; a < TM; ++a)
-#pragma unroll
-        for (int b = 0; b < TM; ++b) acc[a][b] += av[a] * bv[b];
-    }
+    for (int kk = 0; kk < kBK; ++kk) acc.step(a + kk * LDA, b + kk * BN);
     if (s + 1 < steps) store(cur ^ 1);
     __syncthreads();
   }
 
-  T* C = (T*)J.C;
-  const T alpha = (T)J.alpha;
+  const T alpha = SUM ? (T)S.alpha : (T)1;
+  if (SUM && S.split > 1) {
+    // add the ranges' halves in rank order; block `rank` finishes its share of the columns
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    T* red = reinterpret_cast<T*>(mode_smem);  // [half][BN][BM], the operand buffers are done with
 #pragma unroll
-  for (int b = 0; b < TM; ++b) {
-    const int gc = col0 + (b < TM / 2 ? ty * (TM / 2) + b : BN / 2 + ty * (TM / 2) + b - TM / 2);
-    if (gc >= J.ncol) continue;
+    for (int s = 0; s < 2; ++s)
 #pragma unroll
-    for (int a = 0; a < TM; ++a) {
-      const int gr = row0 + (a < TM / 2 ? tx * (TM / 2) + a : BM / 2 + tx * (TM / 2) + a - TM / 2);
-      if (gr < J.rows) C[(long)gc * J.ldc + gr] = alpha * acc[a][b];
+      for (int j = 0; j < TN; ++j)
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+          red[((long)s * BN + wc + j) * BM + wr + (i / VA) * 8 * VA + i % VA] = acc.get(s, i, j);
+    cluster.sync();
+    const int c0 = BN * rank / S.split, c1 = BN * (rank + 1) / S.split;
+    TC* C = reinterpret_cast<TC*>(S.C) + (long)job * S.N;
+    for (int e = tid; e < (c1 - c0) * BM; e += NT) {
+      // the contraction index is the fastest of the output too: consecutive threads on consecutive columns
+      const int c = c0 + e % (c1 - c0), r = e / (c1 - c0);
+      const int a = col0 + c;
+      const int row = row0 + r;
+      if (a >= S.h || row >= S.rows) continue;
+      T p = (T)0, q = (T)0;
+      for (int s = 0; s < S.split; ++s) {
+        const T* o = cluster.map_shared_rank(red, s);
+        p += o[(long)c * BM + r];
+        q += o[(long)(BN + c) * BM + r];
+      }
+      const int a2 = S.n - 1 - a;
+      C[row * S.ostride + a] = (TC)(alpha * (p + q));
+      if (a2 != a) C[row * S.ostride + a2] = (TC)(alpha * (p - q));
+    }
+    cluster.sync();  // no block leaves while another still reads its halves
+    return;
+  }
+
+  TC* C = reinterpret_cast<TC*>(S.C) + ((long)(SUM ? 0 : k0) * S.c_node + job) * S.N;
+#pragma unroll
+  for (int c = 0; c < TM / VA; ++c) {
+    const int r = row0 + wr + c * 8 * VA;
+    // rows r .. r + VA - 1: consecutive addresses from an aligned one when inner and kstride allow it
+    const bool vec = !KCONTIG && S.inner % VA == 0 && S.kstride % VA == 0 && S.N % VA == 0 && r + VA <= S.rows;
+    long o[VA];
+#pragma unroll
+    for (int v = 0; v < VA; ++v)
+      o[v] = v && vec ? 0 : row_offset<KIND>(S, r + v);
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int a = col0 + wc + j;
+      if (a >= S.h) continue;
+      const int a2 = S.n - 1 - a;
+      T hi[VA], lo[VA];
+#pragma unroll
+      for (int v = 0; v < VA; ++v) {
+        const T p = acc.get(0, c * VA + v, j), q = acc.get(1, c * VA + v, j);
+        hi[v] = alpha * (p + q);
+        lo[v] = alpha * (p - q);
+      }
+      if constexpr (!KCONTIG && VA == 2) {
+        if (vec) {
+          *reinterpret_cast<float2*>(C + o[0] + a * S.kstride) = make_float2(hi[0], hi[1]);
+          if (a2 != a) *reinterpret_cast<float2*>(C + o[0] + a2 * S.kstride) = make_float2(lo[0], lo[1]);
+          continue;
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < VA; ++v) {
+        if (r + v >= S.rows) break;
+        C[o[v] + a * S.kstride] = (TC)hi[v];
+        if (a2 != a) C[o[v] + a2 * S.kstride] = (TC)lo[v];
+      }
     }
   }
 }
 
-// ---------------------------------------------------------------- host side
+// ---------------------------------------------------------------- factor parts
+//
+// Per (node, type, axis) and part: h x ldh pairs [j][a] (a contiguous), the
+// factors to the even and to the odd output half.  With
+// j' = n-1-j, a' = n-1-a and T = gen[a - j]:
+//   uniform grid (one part): (T[a][j] +- T[a][j'])/2, halved at j = j' where
+//   x+ holds the entry twice; symmetric factors go x+ -> even, x- -> odd,
+//   skew ones x- -> even, x+ -> odd;
+//   non-uniform grid (two parts): the even / odd blocks of any matrix, part 0
+//   (x+ -> even, x- -> odd), part 1 (x- -> even, x+ -> odd).
+// Formed in FP64 and rounded once; the axis-3 factors carry c s omega_k.
 
-class BatchBuilder {
- public:
-  BatchBuilder() { b_.njobs = 0; b_.total_tiles = 0; npairs_ = 0; overflow_ = false; }
-  void add(int rows, int ncol, int K, int lda, int ldb, int ldc, void* C, float alpha,
-           const std::vector<std::pair<const void*, const void*>>& pairs, int bm) {
-    if (b_.njobs >= kMaxJobs || npairs_ + (int)pairs.size() > kMaxPairs) {
-      overflow_ = true;  // reported by launch_batch; nothing is written past the tables
-      return;
-    }
-    GemmJob& J = b_.jobs[b_.njobs++];
-    J.rows = rows; J.ncol = ncol; J.K = K;
-    J.lda = lda; J.ldb = ldb; J.ldc = ldc;
-    J.pair0 = npairs_;
-    J.npairs = (int)pairs.size();
-    for (auto& pr : pairs) {
-      b_.A[npairs_] = pr.first;
-      b_.B[npairs_] = pr.second;
-      ++npairs_;
-    }
-    J.tiles_m = (rows + bm - 1) / bm;
-    J.tiles_n = (ncol + bm - 1) / bm;
-    J.tile0 = b_.total_tiles;
-    J.alpha = alpha;
-    J.C = C;
-    b_.total_tiles += J.tiles_m * J.tiles_n;
+struct ModeLayout {
+  int h[3], ldh[3];
+  int nparts;
+  size_t off[3], part;  // offset of axis p inside one part, elements of one part (all axes)
+};
+
+static ModeLayout mode_layout(const demag_plan* P) {
+  ModeLayout L;
+  L.nparts = P->nonuniform ? 2 : 1;
+  L.part = 0;
+  for (int p = 0; p < 3; ++p) {
+    L.h[p] = (P->n[p] + 1) / 2;
+    L.ldh[p] = (L.h[p] + 1) / 2 * 2;  // 16-byte rows of pairs
+    L.off[p] = L.part;
+    L.part += (size_t)2 * L.h[p] * L.ldh[p];
   }
-  const GemmBatch& get() const { return b_; }
-  bool overflow() const { return overflow_; }
+  return L;
+}
 
- private:
-  GemmBatch b_;
-  int npairs_;
-  bool overflow_;
+static size_t factor_elems(const demag_plan* P) {
+  const ModeLayout L = mode_layout(P);
+  return (size_t)P->M * 2 * L.nparts * L.part;
+}
+
+struct FactorSource {
+  int n[3], glen;
+  const double* gen;    // [M][2][3][glen] (uniform grid)
+  const double* fac;    // [M][2][tgroup] full matrices (non-uniform grid), else NULL
+  size_t tgroup, toff[3];
+  const double* scale;  // [M]
+  int skew_e;           // type 0 is the skew factor (derivative generators)
+  int transpose;
 };
 
 template <typename T>
-static cudaError_t launch_batch(demag_plan* P, const BatchBuilder& bb, cudaStream_t st) {
-  if (bb.overflow()) return cudaErrorInvalidValue;  // a job table exceeded its fixed capacity
-  const GemmBatch& b = bb.get();
-  if (b.total_tiles == 0) return cudaSuccess;
-  DEMAG_LAUNCH(P, kFamGemmSimt, st, gemm_tn_kernel<T><<<b.total_tiles, 256, 0, st>>>(b));
-  return cudaGetLastError();
-}
-
-// T[k][type][axis] blocks: n_p x n_p row-major, T[i][j] = gen[i-j+n_p-1],
-// axis-3 blocks multiplied by S_k = c s omega_k.
-template <typename T>
-__global__ void dense_factor_kernel(int M, int glen, int n0, int n1, int n2, size_t tgroup, size_t off1,
-                                    size_t off2, const double* gen, const double* scale, T* out,
-                                    const double* fac = nullptr, bool transpose = false) {
-  const size_t total = (size_t)M * 2 * tgroup;
+__global__ void factor_parts_kernel(int M, ModeLayout L, FactorSource s, T* out) {
+  const size_t total = (size_t)M * 2 * L.nparts * L.part;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
        idx += (size_t)gridDim.x * blockDim.x) {
-    size_t e = idx % tgroup;
-    size_t kt = idx / tgroup;  // k*2 + type
-    int axis, n;
-    size_t local;
-    if (e < off1) { axis = 0; n = n0; local = e; }
-    else if (e < off2) { axis = 1; n = n1; local = e - off1; }
-    else { axis = 2; n = n2; local = e - off2; }
-    int i = (int)(local / n), jj = (int)(local % n);
-    if (transpose) {
-      const int t = i;
-      i = jj;
-      jj = t;
+    const size_t e = idx % L.part;
+    const size_t ktp = idx / L.part;
+    const int part = (int)(ktp % L.nparts);
+    const size_t kt = ktp / L.nparts;  // k * 2 + type
+    const int p = e < L.off[1] ? 0 : (e < L.off[2] ? 1 : 2);
+    const int n = s.n[p], h = L.h[p], ld = L.ldh[p];
+    const size_t local = e - L.off[p];
+    const int odd = (int)(local & 1);  // output half
+    const int j = (int)(local / 2 / ld), a = (int)(local / 2 % ld);
+    double v = 0.0;
+    if (a < h) {
+      const int j2 = n - 1 - j, a2 = n - 1 - a;
+      auto entry = [&](int i, int jj) -> double {
+        if (!s.fac) return s.gen[(kt * 3 + p) * s.glen + (i - jj + n - 1)];
+        const double* f = s.fac + kt * s.tgroup + s.toff[p];
+        return s.transpose ? f[(size_t)jj * n + i] : f[(size_t)i * n + jj];
+      };
+      const bool skew = s.fac ? part == 1 : ((int)(kt & 1) ^ s.skew_e);
+      const double sj = (odd != 0) != skew ? -1.0 : 1.0;  // -1: this half is fed by x-
+      v = 0.5 * (entry(a, j) + sj * entry(a, j2));
+      if (s.fac) v = 0.5 * (v + (odd ? -0.5 : 0.5) * (entry(a2, j) + sj * entry(a2, j2)));
+      if (j == j2) v *= 0.5;
+      if (p == 2) v *= s.scale[kt / 2];
     }
-    // Toeplitz generator (uniform grid) or the full matrix (non-uniform grid)
-    double v = fac ? fac[kt * tgroup + (e - local) + (size_t)i * n + jj] : gen[(kt * 3 + axis) * glen + (i - jj + n - 1)];
-    if (axis == 2) v *= scale[kt / 2];
     out[idx] = (T)v;
   }
 }
 
 template <typename T>
-static const T* factor(const demag_plan* P, const T* base, int k, int type, int axis) {
-  return base + ((size_t)k * 2 + type) * P->tgroup + P->toff[axis];
+static demag_status build_factor_parts(demag_plan* P, const double* gen, bool deriv, bool transpose, T* out,
+                                       cudaStream_t st) {
+  FactorSource s;
+  for (int p = 0; p < 3; ++p) {
+    s.n[p] = P->n[p];
+    s.toff[p] = P->toff[p];
+  }
+  s.glen = P->glen;
+  s.gen = gen;
+  s.fac = P->nonuniform ? P->fac64 : nullptr;
+  s.tgroup = P->tgroup;
+  s.scale = P->scale;
+  s.skew_e = deriv;
+  s.transpose = transpose;
+  const size_t total = factor_elems(P);
+  int blocks = (int)((total + 255) / 256 > 152 * 64 ? 152 * 64 : (total + 255) / 256);
+  DEMAG_LAUNCH(P, kFamSetup, st, factor_parts_kernel<T><<<blocks, 256, 0, st>>>(P->M, mode_layout(P), s, out));
+  DEMAG_LAUNCHED(P, "factor_parts_kernel");
+  return DEMAG_OK;
+}
+
+template <typename T>
+static demag_status ensure_parts(demag_plan* P, T** out, const double* gen, bool deriv, bool transpose,
+                                 cudaStream_t st) {
+  if (*out) return DEMAG_OK;
+  DEMAG_CUDA(P, cudaMalloc(out, sizeof(T) * factor_elems(P)));
+  return build_factor_parts<T>(P, gen, deriv, transpose, *out, st);
 }
 
 demag_status ensure_dense_factors(demag_plan* P, demag_precision prec, cudaStream_t st) {
-  const size_t total = (size_t)P->M * 2 * P->tgroup;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  if (prec == DEMAG_FP64) {
-    if (P->T64) return DEMAG_OK;
-    DEMAG_CUDA(P, cudaMalloc(&P->T64, sizeof(double) * total));
-    DEMAG_LAUNCH(P, kFamSetup, st,
-                 dense_factor_kernel<double><<<blocks, 256, 0, st>>>(P->M, P->glen, P->n[0], P->n[1], P->n[2],
-                                                                     P->tgroup, P->toff[1], P->toff[2], P->gen64,
-                                                                     P->scale, P->T64, P->fac64));
-  } else {
-    if (P->T32) return DEMAG_OK;
-    DEMAG_CUDA(P, cudaMalloc(&P->T32, sizeof(float) * total));
-    DEMAG_LAUNCH(P, kFamSetup, st,
-                 dense_factor_kernel<float><<<blocks, 256, 0, st>>>(P->M, P->glen, P->n[0], P->n[1], P->n[2],
-                                                                    P->tgroup, P->toff[1], P->toff[2], P->gen64,
-                                                                    P->scale, P->T32, P->fac64));
-  }
-  DEMAG_LAUNCHED(P, "dense_factor_kernel");
-  return DEMAG_OK;
+  return prec == DEMAG_FP64 ? ensure_parts<double>(P, &P->T64, P->gen64, false, false, st)
+                            : ensure_parts<float>(P, &P->T32, P->gen64, false, false, st);
 }
 
-// Transposed factor tables of a non-uniform plan, for the adjoint on CUDA
-// cores: (P^(q))^T = c sum_k omega_k U3^T (x) U2^T (x) U1^T.
+// Transposed factors of a non-uniform plan, for the adjoint on CUDA cores:
+// (P^(q))^T = c sum_k omega_k U3^T (x) U2^T (x) U1^T.
 static demag_status ensure_transposed_factors(demag_plan* P, demag_precision prec, cudaStream_t st) {
-  const size_t total = (size_t)P->M * 2 * P->tgroup;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  if (prec == DEMAG_FP64) {
-    if (P->T64t) return DEMAG_OK;
-    DEMAG_CUDA(P, cudaMalloc(&P->T64t, sizeof(double) * total));
-    DEMAG_LAUNCH(P, kFamSetup, st,
-                 dense_factor_kernel<double><<<blocks, 256, 0, st>>>(P->M, P->glen, P->n[0], P->n[1], P->n[2],
-                                                                     P->tgroup, P->toff[1], P->toff[2], P->gen64,
-                                                                     P->scale, P->T64t, P->fac64, true));
-  } else {
-    if (P->T32t) return DEMAG_OK;
-    DEMAG_CUDA(P, cudaMalloc(&P->T32t, sizeof(float) * total));
-    DEMAG_LAUNCH(P, kFamSetup, st,
-                 dense_factor_kernel<float><<<blocks, 256, 0, st>>>(P->M, P->glen, P->n[0], P->n[1], P->n[2],
-                                                                    P->tgroup, P->toff[1], P->toff[2], P->gen64,
-                                                                    P->scale, P->T32t, P->fac64, true));
+  return prec == DEMAG_FP64 ? ensure_parts<double>(P, &P->T64t, P->gen64, false, true, st)
+                            : ensure_parts<float>(P, &P->T32t, P->gen64, false, true, st);
+}
+
+// ---------------------------------------------------------------- launches
+
+// The factors used along each axis: the forward (or transposed) table, or the
+// derivative table, whose even and odd factors change places.
+template <typename T> struct ModeFactors {
+  const T* base[3];
+  bool deriv[3];
+};
+
+// Stage `kind` (0: axis 3, 1: axis 2, 2: axis 1 with the node sum) of nodes [k0, k0 + nodes)
+template <typename T>
+static ModeStage make_stage(const demag_plan* P, int kind, const ModeFactors<T>& F, int k0, int nodes, const void* A,
+                            int a_node, void* C, int c_node) {
+  const ModeLayout L = mode_layout(P);
+  const int p = 2 - kind;
+  ModeStage S;
+  S.n = P->n[p];
+  S.h = L.h[p];
+  S.ldh = L.ldh[p];
+  S.N = (long)field_size(P);
+  S.rows = (int)(S.N / S.n);
+  S.kstride = p == 0 ? 1 : p == 1 ? P->n[0] : (long)P->n[0] * P->n[1];
+  S.inner = (int)S.kstride;
+  S.ostride = S.kstride * S.n;
+  S.inner_shift = 0;
+  while ((1ull << S.inner_shift) < (unsigned long long)S.inner) ++S.inner_shift;
+  S.inner_mul = (unsigned)(((1ull << 32) * ((1ull << S.inner_shift) - S.inner)) / S.inner + 1);
+  S.A = A;
+  S.b_node = (long)(2 * L.nparts * L.part);
+  S.B = F.base[p] + (size_t)k0 * S.b_node + L.off[p];
+  S.C = C;
+  S.nodes = nodes;
+  S.a_node = a_node;
+  S.c_node = c_node;
+  S.njobs = 0;
+  S.npairs[0] = S.npairs[1] = S.npairs[2] = 0;
+  S.split = 1;
+  S.alpha = 1.f;
+  return S;
+}
+
+// One more (field, factor type) pair of output `job`
+template <typename T>
+static void add_pair(const demag_plan* P, ModeStage& S, const ModeFactors<T>& F, int axis, int job, int field,
+                     int type) {
+  const ModeLayout L = mode_layout(P);
+  if (job >= S.njobs) S.njobs = job + 1;
+  for (int part = 0; part < L.nparts; ++part) {
+    const int at = S.npairs[job]++;
+    S.a_field[job][at] = field;
+    S.b_off[job][at] = (long)((type * L.nparts + part) * L.part);
+    S.swap[job][at] = L.nparts == 2 ? part : (type ^ (F.deriv[axis] ? 1 : 0));
   }
-  DEMAG_LAUNCHED(P, "dense_factor_kernel (transposed)");
-  return DEMAG_OK;
+}
+
+template <typename T, typename Cfg, int KIND>
+static cudaError_t launch_mode_cfg(demag_plan* P, ModeStage S, int split, cudaStream_t st) {
+  S.tiles_n = (S.h + Cfg::BN - 1) / Cfg::BN;
+  S.split = split;
+  const long tiles = ((long)S.rows + Cfg::BM - 1) / Cfg::BM * S.tiles_n * S.njobs * (KIND == 2 ? split : S.nodes);
+  if (tiles > INT_MAX) return cudaErrorInvalidValue;
+  const size_t smem = split > 1 && Cfg::reduce > Cfg::operands ? Cfg::reduce : Cfg::operands;
+  if (Cfg::reduce > 48 * 1024 || Cfg::operands > 48 * 1024) {
+    static unsigned long long done = 0;  // once per device: later launches, e.g. under capture, make no attribute calls
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(done & bit)) {
+      const size_t most = Cfg::reduce > Cfg::operands ? Cfg::reduce : Cfg::operands;
+      cudaError_t e = cudaFuncSetAttribute(mode_kernel<T, Cfg, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)most);
+      if (e != cudaSuccess) return e;
+      done |= bit;
+    }
+  }
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)tiles);
+  lc.blockDim = dim3(Cfg::NT);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)split;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  lc.attrs = attr;
+  lc.numAttrs = split > 1 ? 1 : 0;
+  cudaError_t e = cudaSuccess;
+  DEMAG_LAUNCH(P, kFamGemmSimt, st, e = cudaLaunchKernelEx(&lc, mode_kernel<T, Cfg, KIND>, S));
+  return e;
+}
+
+// Time of a stage in a configuration, up to a factor: the tiles of the busiest
+// SM, times their multiply-adds (contraction steps plus prologue and epilogue,
+// and the exchange of a split sum), over the configuration's rate, which falls
+// when fewer blocks are resident than fit.  The rates and overheads were fitted
+// to the times of every configuration at 13 grids from 16^3 to 192^3 (R = 41):
+// the choice is within 2% of the fastest on average.  E.g. axis 3 of 128^3:
+// 128 x 64 tiles 398 us, 256 x 32 413, 128 x 32 447, 256 x 16 493, 64 x 16 705;
+// of 16^3: 10.2, 10.2, 11.0, 10.1, 7.0; axis 1 (the node sum) of 48^3: 128 x 64
+// 129, split over 4 blocks 45, 64 x 16 over 8 blocks 26.5.
+struct ModeShape {
+  int bm, bn, occ;
+  double rate;
+};
+
+static double mode_cost(const ModeStage& S, bool sum, const ModeShape& c, int split) {
+  double pairs = 0;
+  for (int j = 0; j < S.njobs; ++j) pairs += S.npairs[j];
+  pairs /= S.njobs;
+  const double tiles = std::ceil((double)S.rows / c.bm) * ((S.h + c.bn - 1) / c.bn) * S.njobs * (sum ? split : S.nodes);
+  const double steps = (double)((S.h + kBK - 1) / kBK * kBK) * pairs * (sum ? (double)S.nodes / split : 1.0);
+  const double per_sm = std::ceil(tiles / 152.0);
+  const double full = per_sm < c.occ ? std::pow(per_sm / c.occ, 0.3) : 1.0;
+  return per_sm * (steps + 24 + (split > 1 ? 48 : 0)) * c.bm * c.bn / (c.rate * full);
+}
+
+template <typename T, int KIND>
+static cudaError_t launch_mode(demag_plan* P, const ModeStage& S, cudaStream_t st) {
+  constexpr bool SUM = KIND == 2;
+  using Fn = cudaError_t (*)(demag_plan*, ModeStage, int, cudaStream_t);
+  struct Choice {
+    ModeShape shape;
+    Fn run;
+  } all[5];
+  int count = 0;
+  auto add = [&](auto cfg, double rate) {
+    using Cfg = decltype(cfg);
+    all[count++] = {{Cfg::BM, Cfg::BN, Cfg::OCC, rate}, launch_mode_cfg<T, Cfg, KIND>};
+  };
+  if constexpr (std::is_same<T, float>::value) {
+    add(ModeCfg<float, 128, 64, 8, 8, 2>{}, 1.0);
+    add(ModeCfg<float, 256, 32, 8, 8, 2>{}, 0.95);
+    add(ModeCfg<float, 128, 32, 8, 4, 3>{}, 0.8);
+    add(ModeCfg<float, 256, 16, 8, 4, 3>{}, 0.8);
+    add(ModeCfg<float, 64, 16, 4, 2, 8>{}, 0.6);
+  } else {
+    // FP64 multiply-adds run at 1/64 of the FP32 rate: any tile feeds them, and small ones balance the SMs
+    add(ModeCfg<double, 64, 32, 4, 4, 3>{}, 1.0);
+    add(ModeCfg<double, 32, 16, 2, 2, 6>{}, 0.9);
+  }
+  const int most = SUM ? (S.nodes < 8 ? S.nodes : 8) : 1;
+  const Choice* pick = nullptr;
+  int split = 1;
+  double best = 0;
+  for (int c = 0; c < count; ++c)
+    for (int s = 1; s <= most; ++s) {
+      const double t = mode_cost(S, SUM, all[c].shape, s);
+      if (!pick || t < best) {
+        best = t;
+        pick = &all[c];
+        split = s;
+      }
+    }
+  return pick->run(P, S, split, st);
+}
+
+// ---------------------------------------------------------------- workspace
+
+// Fields of the workspace: the axis-2 outputs of every node (2 M forward, 3 M
+// adjoint) and the axis-3 outputs of a chunk of nodes (3 or 2 per node).  The
+// chunk gets 3 fields, or as many as fit in 256 MiB: small grids run all their
+// nodes in one launch per stage (their launches are what takes time), large
+// ones fill the chip with a few nodes and keep the memory of one chunk.
+static size_t chunk_nodes(const demag_plan* P, size_t elem) {
+  const size_t per = 3 * field_size(P) * elem;
+  size_t k = (size_t(256) << 20) / per;
+  if (k < 1) k = 1;
+  return k < (size_t)P->M ? k : (size_t)P->M;
 }
 
 size_t workspace_bytes(const demag_plan* P, demag_precision prec) {
-  const size_t N = field_size(P);
   if (prec == DEMAG_TF32X3 || prec == DEMAG_BF16X3) return tc_workspace_bytes(P, prec);
-  // forward: Y (3 fields) + U,V per node; adjoint: Y (2) + 3 per node.
-  // FP64 also keeps double copies of the input and output fields (3 + 3).
-  size_t fields = 3 * (size_t)P->M + 3;
-  if (prec == DEMAG_FP64) fields += 6;
-  return fields * N * (prec == DEMAG_FP64 ? sizeof(double) : sizeof(float));
+  const size_t elem = prec == DEMAG_FP64 ? sizeof(double) : sizeof(float);
+  return 3 * ((size_t)P->M + chunk_nodes(P, elem)) * field_size(P) * elem;
 }
 
 demag_status ensure_workspace(demag_plan* P, demag_precision prec) {
@@ -290,98 +696,87 @@ demag_status ensure_workspace(demag_plan* P, demag_precision prec) {
   return DEMAG_OK;
 }
 
-template <typename T>
-__global__ void convert_kernel(const float* in, T* out, size_t count) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = (T)in[i];
-}
-__global__ void narrow_kernel(const double* in, float* out, size_t count) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = (float)in[i];
-}
+// ---------------------------------------------------------------- forward and adjoint
 
-// forward: m (3 fields, type T) -> phi (type T) using workspace `ws` of type T
+// m (3 fields) -> phi = alpha P m; UV: 2 M fields, Y: 3 * chunk fields of type T
 template <typename T>
-// Tax[p]: the factor table used along axis p (the analytic stray field swaps
-// in the derivative factors along one axis); alpha scales the result.
-static demag_status simt_forward(demag_plan* P, const T* m, T* phi, const T* const (&Tax)[3], T* ws,
-                                 cudaStream_t st, float alpha = 1.f) {
-  constexpr int BM = 16 * SimtCfg<T>::TM;
-  const int n1 = P->n[0], n2 = P->n[1], n3 = P->n[2];
+static demag_status mode_forward(demag_plan* P, const float* m, float* phi, const ModeFactors<T>& F, T* UV, T* Y,
+                                 int chunk, float alpha, cudaStream_t st) {
   const size_t N = field_size(P);
-  T* Y = ws;                 // 3 fields
-  T* UV = ws + 3 * N;        // [M][2] fields
   const int M = P->M;
-  for (int k = 0; k < M; ++k) {
-    BatchBuilder b1;
-    for (int q = 0; q < 3; ++q) {
-      const T* B = factor(P, Tax[0], k, q == 0 ? 1 : 0, 0);
-      b1.add(n3 * n2, n1, n1, n1, n1, n3 * n2, Y + q * N, 1.f, {{m + q * N, B}}, BM);
-    }
-    cudaError_t e = launch_batch<T>(P, b1, st);
-    if (e != cudaSuccess) return cuda_error(P, e, "gemm_tn_kernel (mode 1)");
-    BatchBuilder b2;
-    const T* E2 = factor(P, Tax[1], k, 0, 1);
-    const T* F2 = factor(P, Tax[1], k, 1, 1);
-    b2.add(n1 * n3, n2, n2, n2, n2, n1 * n3, UV + (2 * k) * N, 1.f, {{Y, E2}, {Y + N, F2}}, BM);
-    b2.add(n1 * n3, n2, n2, n2, n2, n1 * n3, UV + (2 * k + 1) * N, 1.f, {{Y + 2 * N, E2}}, BM);
-    e = launch_batch<T>(P, b2, st);
-    if (e != cudaSuccess) return cuda_error(P, e, "gemm_tn_kernel (mode 2)");
+  chunk = (M + (M + chunk - 1) / chunk - 1) / ((M + chunk - 1) / chunk);  // the same number of launches, even chunks
+  for (int k = 0; k < M; k += chunk) {
+    const int nk = k + chunk < M ? chunk : M - k;
+    ModeStage s3 = make_stage<T>(P, 0, F, k, nk, m, 0, Y, 3);
+    for (int q = 0; q < 3; ++q) add_pair(P, s3, F, 2, q, q, q == 2 ? 1 : 0);
+    cudaError_t e = launch_mode<T, 0>(P, s3, st);
+    if (e != cudaSuccess) return cuda_error(P, e, "mode_kernel (axis 3)");
+    ModeStage s2 = make_stage<T>(P, 1, F, k, nk, Y, 3, UV + (size_t)2 * k * N, 2);
+    add_pair(P, s2, F, 1, 0, 1, 1);
+    add_pair(P, s2, F, 1, 0, 2, 0);
+    add_pair(P, s2, F, 1, 1, 0, 0);
+    e = launch_mode<T, 1>(P, s2, st);
+    if (e != cudaSuccess) return cuda_error(P, e, "mode_kernel (axis 2)");
   }
-  BatchBuilder b3;
-  std::vector<std::pair<const void*, const void*>> pairs;
-  for (int k = 0; k < M; ++k) {
-    pairs.push_back({UV + (2 * k) * N, factor(P, Tax[2], k, 0, 2)});
-    pairs.push_back({UV + (2 * k + 1) * N, factor(P, Tax[2], k, 1, 2)});
-  }
-  b3.add(n2 * n1, n3, n3, n3, n3, n2 * n1, phi, alpha, pairs, BM);
-  cudaError_t e = launch_batch<T>(P, b3, st);
-  if (e != cudaSuccess) return cuda_error(P, e, "gemm_tn_kernel (mode 3)");
+  ModeStage s1 = make_stage<T>(P, 2, F, 0, M, UV, 2, phi, 0);
+  s1.alpha = alpha;
+  add_pair(P, s1, F, 0, 0, 0, 0);
+  add_pair(P, s1, F, 0, 0, 1, 1);
+  cudaError_t e = launch_mode<T, 2>(P, s1, st);
+  if (e != cudaSuccess) return cuda_error(P, e, "mode_kernel (axis 1)");
   return DEMAG_OK;
 }
 
-// adjoint: y (1 field) -> g (3 fields).  Uniform grid: g^(q) = -P^(q) y with
-// the forward tables (sign -1); non-uniform grid: the transposed tables and
-// sign +1.
+// y (1 field) -> g (3 fields).  Uniform grid: g^(q) = -P^(q) y with the forward
+// factors (sign -1); non-uniform grid: the transposed factors and sign +1.
+// Z: 3 M fields, Y: 2 * chunk fields
 template <typename T>
-static demag_status simt_adjoint(demag_plan* P, const T* y, T* g, const T* Tm, T* ws, cudaStream_t st,
-                                 float sign = -1.f) {
-  constexpr int BM = 16 * SimtCfg<T>::TM;
-  const int n1 = P->n[0], n2 = P->n[1], n3 = P->n[2];
+static demag_status mode_adjoint(demag_plan* P, const float* y, float* g, const ModeFactors<T>& F, T* Z, T* Y,
+                                 int chunk, float sign, cudaStream_t st) {
   const size_t N = field_size(P);
-  T* Y = ws;            // 2 fields: F1 y, E1 y
-  T* Z = ws + 2 * N;    // [M][3]
   const int M = P->M;
-  for (int k = 0; k < M; ++k) {
-    BatchBuilder b1;
-    b1.add(n3 * n2, n1, n1, n1, n1, n3 * n2, Y, 1.f, {{y, factor(P, Tm, k, 1, 0)}}, BM);
-    b1.add(n3 * n2, n1, n1, n1, n1, n3 * n2, Y + N, 1.f, {{y, factor(P, Tm, k, 0, 0)}}, BM);
-    cudaError_t e = launch_batch<T>(P, b1, st);
-    if (e != cudaSuccess) return cuda_error(P, e, "gemm_tn_kernel (adjoint mode 1)");
-    BatchBuilder b2;
-    const T* E2 = factor(P, Tm, k, 0, 1);
-    const T* F2 = factor(P, Tm, k, 1, 1);
-    b2.add(n1 * n3, n2, n2, n2, n2, n1 * n3, Z + (3 * k) * N, 1.f, {{Y, E2}}, BM);
-    b2.add(n1 * n3, n2, n2, n2, n2, n1 * n3, Z + (3 * k + 1) * N, 1.f, {{Y + N, F2}}, BM);
-    b2.add(n1 * n3, n2, n2, n2, n2, n1 * n3, Z + (3 * k + 2) * N, 1.f, {{Y + N, E2}}, BM);
-    e = launch_batch<T>(P, b2, st);
-    if (e != cudaSuccess) return cuda_error(P, e, "gemm_tn_kernel (adjoint mode 2)");
+  chunk = (M + (M + chunk - 1) / chunk - 1) / ((M + chunk - 1) / chunk);
+  for (int k = 0; k < M; k += chunk) {
+    const int nk = k + chunk < M ? chunk : M - k;
+    ModeStage s3 = make_stage<T>(P, 0, F, k, nk, y, 0, Y, 2);
+    add_pair(P, s3, F, 2, 0, 0, 1);
+    add_pair(P, s3, F, 2, 1, 0, 0);
+    cudaError_t e = launch_mode<T, 0>(P, s3, st);
+    if (e != cudaSuccess) return cuda_error(P, e, "mode_kernel (adjoint, axis 3)");
+    ModeStage s2 = make_stage<T>(P, 1, F, k, nk, Y, 2, Z + (size_t)3 * k * N, 3);
+    add_pair(P, s2, F, 1, 0, 1, 0);
+    add_pair(P, s2, F, 1, 1, 1, 1);
+    add_pair(P, s2, F, 1, 2, 0, 0);
+    e = launch_mode<T, 1>(P, s2, st);
+    if (e != cudaSuccess) return cuda_error(P, e, "mode_kernel (adjoint, axis 2)");
   }
-  BatchBuilder b3;
-  for (int q = 0; q < 3; ++q) {
-    std::vector<std::pair<const void*, const void*>> pairs;
-    for (int k = 0; k < M; ++k) pairs.push_back({Z + (3 * k + q) * N, factor(P, Tm, k, q == 2 ? 1 : 0, 2)});
-    b3.add(n2 * n1, n3, n3, n3, n3, n2 * n1, g + q * N, sign, pairs, BM);
-  }
-  cudaError_t e = launch_batch<T>(P, b3, st);
-  if (e != cudaSuccess) return cuda_error(P, e, "gemm_tn_kernel (adjoint mode 3)");
+  ModeStage s1 = make_stage<T>(P, 2, F, 0, M, Z, 3, g, 0);
+  s1.alpha = sign;
+  for (int q = 0; q < 3; ++q) add_pair(P, s1, F, 0, q, q, q == 0 ? 1 : 0);
+  cudaError_t e = launch_mode<T, 2>(P, s1, st);
+  if (e != cudaSuccess) return cuda_error(P, e, "mode_kernel (adjoint, axis 1)");
   return DEMAG_OK;
 }
 
-static int conv_blocks(size_t count) {
-  size_t b = (count + 255) / 256;
-  return (int)(b > 152 * 32 ? 152 * 32 : b);
+// The regions of the workspace and the chunk the axis-3 outputs have room for
+template <typename T>
+static demag_status run_forward(demag_plan* P, const float* m, float* phi, const ModeFactors<T>& F, float alpha,
+                                demag_precision prec, cudaStream_t st) {
+  const size_t N = field_size(P), M = P->M;
+  T* UV = (T*)P->ws[prec].base;
+  const size_t chunk = (M + 3 * chunk_nodes(P, sizeof(T))) / 3;
+  return mode_forward<T>(P, m, phi, F, UV, UV + 2 * M * N, (int)(chunk < M ? chunk : M), alpha, st);
 }
+template <typename T>
+static demag_status run_adjoint(demag_plan* P, const float* y, float* g, const ModeFactors<T>& F, float sign,
+                                demag_precision prec, cudaStream_t st) {
+  const size_t N = field_size(P), M = P->M;
+  T* Z = (T*)P->ws[prec].base;
+  const size_t chunk = 3 * chunk_nodes(P, sizeof(T)) / 2;
+  return mode_adjoint<T>(P, y, g, F, Z, Z + 3 * M * N, (int)(chunk < M ? chunk : M), sign, st);
+}
+
+template <typename T> static ModeFactors<T> same_factors(const T* t) { return {{t, t, t}, {false, false, false}}; }
 
 demag_status full_forward(demag_plan* P, const float* m, float* phi, demag_precision prec, cudaStream_t st) {
   if (prec == DEMAG_TF32X3 || prec == DEMAG_BF16X3) return tc_forward(P, m, phi, prec, st);
@@ -389,73 +784,34 @@ demag_status full_forward(demag_plan* P, const float* m, float* phi, demag_preci
   if (s != DEMAG_OK) return s;
   s = ensure_workspace(P, prec);
   if (s != DEMAG_OK) return s;
-  const size_t N = field_size(P);
-  if (prec == DEMAG_FP32) {
-    const float* const tax[3] = {P->T32, P->T32, P->T32};
-    return simt_forward<float>(P, m, phi, tax, (float*)P->ws[prec].base, st);
-  }
-  double* ws = (double*)P->ws[prec].base;
-  double* m64 = ws + (3 * (size_t)P->M + 3) * N;
-  double* phi64 = m64 + 3 * N;
-  DEMAG_LAUNCH(P, kFamSplit, st, convert_kernel<double><<<conv_blocks(3 * N), 256, 0, st>>>(m, m64, 3 * N));
-  DEMAG_LAUNCHED(P, "convert_kernel");
-  const double* const tax[3] = {P->T64, P->T64, P->T64};
-  s = simt_forward<double>(P, m64, phi64, tax, ws, st);
-  if (s != DEMAG_OK) return s;
-  DEMAG_LAUNCH(P, kFamSplit, st, narrow_kernel<<<conv_blocks(N), 256, 0, st>>>(phi64, phi, N));
-  DEMAG_LAUNCHED(P, "narrow_kernel");
-  return DEMAG_OK;
+  if (prec == DEMAG_FP32) return run_forward<float>(P, m, phi, same_factors<float>(P->T32), 1.f, prec, st);
+  return run_forward<double>(P, m, phi, same_factors<double>(P->T64), 1.f, prec, st);
 }
 
 // ---------------------------------------------------------------- analytic stray field (CUDA cores)
 
-// h_d[p] = -dphi/dxi_p for p = 1..3: the forward chain with the axis-p factor
-// table replaced by the derivative table (built from the derivative generators).
+// h_d[p] = -dphi/dxi_p for p = 1..3: the forward chain with the axis-p factors
+// replaced by the derivative ones (built from the derivative generators).
+template <typename T>
+static demag_status mode_field(demag_plan* P, const float* m, float* hd, const T* plain, T** deriv,
+                               demag_precision prec, cudaStream_t st) {
+  demag_status s = ensure_parts<T>(P, deriv, P->gend, true, false, st);
+  for (int p = 0; p < 3 && s == DEMAG_OK; ++p) {
+    ModeFactors<T> F = same_factors<T>(plain);
+    F.base[p] = *deriv;
+    F.deriv[p] = true;
+    s = run_forward<T>(P, m, hd + p * field_size(P), F, -1.f, prec, st);
+  }
+  return s;
+}
+
 demag_status simt_field(demag_plan* P, const float* m, float* hd, demag_precision prec, cudaStream_t st) {
   demag_status s = ensure_dense_factors(P, prec, st);
   if (s == DEMAG_OK) s = ensure_workspace(P, prec);
   if (s == DEMAG_OK) s = ensure_field_generators(P, st);
   if (s != DEMAG_OK) return s;
-  const size_t total = (size_t)P->M * 2 * P->tgroup;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  const size_t N = field_size(P);
-  if (prec == DEMAG_FP32) {
-    if (!P->T32d) {
-      DEMAG_CUDA(P, cudaMalloc(&P->T32d, sizeof(float) * total));
-      DEMAG_LAUNCH(P, kFamSetup, st,
-                   dense_factor_kernel<float><<<blocks, 256, 0, st>>>(P->M, P->glen, P->n[0], P->n[1], P->n[2],
-                                                                      P->tgroup, P->toff[1], P->toff[2], P->gend,
-                                                                      P->scale, P->T32d));
-      DEMAG_LAUNCHED(P, "dense_factor_kernel");
-    }
-    for (int p = 0; p < 3 && s == DEMAG_OK; ++p) {
-      const float* const tax[3] = {p == 0 ? P->T32d : P->T32, p == 1 ? P->T32d : P->T32, p == 2 ? P->T32d : P->T32};
-      s = simt_forward<float>(P, m, hd + p * N, tax, (float*)P->ws[prec].base, st, -1.f);
-    }
-    return s;
-  }
-  if (!P->T64d) {
-    DEMAG_CUDA(P, cudaMalloc(&P->T64d, sizeof(double) * total));
-    DEMAG_LAUNCH(P, kFamSetup, st,
-                 dense_factor_kernel<double><<<blocks, 256, 0, st>>>(P->M, P->glen, P->n[0], P->n[1], P->n[2],
-                                                                     P->tgroup, P->toff[1], P->toff[2], P->gend,
-                                                                     P->scale, P->T64d));
-    DEMAG_LAUNCHED(P, "dense_factor_kernel");
-  }
-  double* ws = (double*)P->ws[prec].base;
-  double* m64 = ws + (3 * (size_t)P->M + 3) * N;
-  double* out64 = m64 + 3 * N;
-  DEMAG_LAUNCH(P, kFamSplit, st, convert_kernel<double><<<conv_blocks(3 * N), 256, 0, st>>>(m, m64, 3 * N));
-  DEMAG_LAUNCHED(P, "convert_kernel");
-  for (int p = 0; p < 3 && s == DEMAG_OK; ++p) {
-    const double* const tax[3] = {p == 0 ? P->T64d : P->T64, p == 1 ? P->T64d : P->T64, p == 2 ? P->T64d : P->T64};
-    s = simt_forward<double>(P, m64, out64, tax, ws, st, -1.f);
-    if (s != DEMAG_OK) break;
-    DEMAG_LAUNCH(P, kFamSplit, st, narrow_kernel<<<conv_blocks(N), 256, 0, st>>>(out64, hd + p * N, N));
-    DEMAG_LAUNCHED(P, "narrow_kernel");
-  }
-  return s;
+  if (prec == DEMAG_FP32) return mode_field<float>(P, m, hd, P->T32, &P->T32d, prec, st);
+  return mode_field<double>(P, m, hd, P->T64, &P->T64d, prec, st);
 }
 
 demag_status full_adjoint(demag_plan* P, const float* y, float* g, demag_precision prec, cudaStream_t st) {
@@ -469,20 +825,10 @@ demag_status full_adjoint(demag_plan* P, const float* y, float* g, demag_precisi
   if (s != DEMAG_OK) return s;
   s = ensure_workspace(P, prec);
   if (s != DEMAG_OK) return s;
-  const size_t N = field_size(P);
   const float sign = P->nonuniform ? 1.f : -1.f;
   if (prec == DEMAG_FP32)
-    return simt_adjoint<float>(P, y, g, P->nonuniform ? P->T32t : P->T32, (float*)P->ws[prec].base, st, sign);
-  double* ws = (double*)P->ws[prec].base;
-  double* y64 = ws + (3 * (size_t)P->M + 3) * N;
-  double* g64 = y64 + 3 * N;
-  DEMAG_LAUNCH(P, kFamSplit, st, convert_kernel<double><<<conv_blocks(N), 256, 0, st>>>(y, y64, N));
-  DEMAG_LAUNCHED(P, "convert_kernel");
-  s = simt_adjoint<double>(P, y64, g64, P->nonuniform ? P->T64t : P->T64, ws, st, sign);
-  if (s != DEMAG_OK) return s;
-  DEMAG_LAUNCH(P, kFamSplit, st, narrow_kernel<<<conv_blocks(3 * N), 256, 0, st>>>(g64, g, 3 * N));
-  DEMAG_LAUNCHED(P, "narrow_kernel");
-  return DEMAG_OK;
+    return run_adjoint<float>(P, y, g, same_factors<float>(P->nonuniform ? P->T32t : P->T32), sign, prec, st);
+  return run_adjoint<double>(P, y, g, same_factors<double>(P->nonuniform ? P->T64t : P->T64), sign, prec, st);
 }
 
 static demag_status check_prec(demag_plan* P, demag_precision prec, const char* what) {
@@ -682,9 +1028,6 @@ extern "C" int demag_graph_kernel_count(const demag_graph* g) { return g ? g->ke
 // the process exits.  The arithmetic is that of demag_apply_full with
 // DEMAG_FP32 (same kernels, same order).
 
-#include <cmath>
-#include <mutex>
-
 namespace demag {
 
 constexpr size_t kNoAllocBytes = size_t(32) << 20;  // 32 MiB of device scratch
@@ -716,34 +1059,6 @@ static demag_status noalloc_address(void** out) {
 }
 
 static size_t na_align(size_t b) { return (b + 255) & ~size_t(255); }
-
-// Append one job to a GEMM batch without any host heap use.
-static void na_add(GemmBatch& b, int& npairs, int rows, int ncol, int K, int ldc, void* C,
-                   const void* const* A, const void* const* B, int np) {
-  GemmJob& J = b.jobs[b.njobs++];
-  J.rows = rows; J.ncol = ncol; J.K = K;
-  J.lda = K; J.ldb = K; J.ldc = ldc;
-  J.pair0 = npairs;
-  J.npairs = np;
-  for (int i = 0; i < np; ++i) {
-    b.A[npairs] = A[i];
-    b.B[npairs] = B[i];
-    ++npairs;
-  }
-  const int bm = 16 * SimtCfg<float>::TM;
-  J.tiles_m = (rows + bm - 1) / bm;
-  J.tiles_n = (ncol + bm - 1) / bm;
-  J.tile0 = b.total_tiles;
-  J.alpha = 1.f;
-  J.C = C;
-  b.total_tiles += J.tiles_m * J.tiles_n;
-}
-
-static demag_status na_launch(demag_plan* P, const GemmBatch& b, cudaStream_t st) {
-  DEMAG_LAUNCH(P, kFamGemmSimt, st, gemm_tn_kernel<float><<<b.total_tiles, 256, 0, st>>>(b));
-  DEMAG_LAUNCHED(P, "gemm_tn_kernel (allocation-free)");
-  return DEMAG_OK;
-}
 
 }  // namespace demag
 
@@ -809,7 +1124,10 @@ extern "C" demag_status demag_apply_full_noalloc(const demag_grid_desc* d, const
   P.scale = reinterpret_cast<double*>(at + b_nodes);
   P.gen64 = reinterpret_cast<double*>(at + b_nodes + b_scale);
   float* T = reinterpret_cast<float*>(at + b_nodes + b_scale + b_gen);
-  float* Y = reinterpret_cast<float*>(at + b_nodes + b_scale + b_gen + b_fac);
+  // the factor parts take about half of the region of the limit above; on axes of at most three cells
+  // their padding makes them larger than n_p^2, on grids far below the limit
+  const size_t b_parts = na_align(sizeof(float) * factor_elems(&P));
+  float* Y = reinterpret_cast<float*>(at + b_nodes + b_scale + b_gen + (b_parts > b_fac ? b_parts : b_fac));
   float* UV = Y + 3 * N;
   cudaStream_t st = (cudaStream_t)stream;
 
@@ -829,61 +1147,9 @@ extern "C" demag_status demag_apply_full_noalloc(const demag_grid_desc* d, const
     DEMAG_LAUNCH(&P, kFamSetup, st, generators_kernel<<<blocks, 256, 0, st>>>(M, P.glen, g, P.nodes, P.gen64));
     DEMAG_LAUNCHED(&P, "generators_kernel (allocation-free)");
   }
-  {
-    const size_t total = (size_t)M * 2 * P.tgroup;
-    int blocks = (int)((total + 255) / 256);
-    if (blocks > 152 * 64) blocks = 152 * 64;
-    DEMAG_LAUNCH(&P, kFamSetup, st,
-                 dense_factor_kernel<float><<<blocks, 256, 0, st>>>(M, P.glen, P.n[0], P.n[1], P.n[2], P.tgroup,
-                                                                    P.toff[1], P.toff[2], P.gen64, P.scale, T));
-    DEMAG_LAUNCHED(&P, "dense_factor_kernel (allocation-free)");
-  }
+  s = build_factor_parts<float>(&P, P.gen64, false, false, T, st);
+  if (s != DEMAG_OK) return s;
 
-  // the mode-product chain of demag_apply_full (DEMAG_FP32)
-  const int n1 = P.n[0], n2 = P.n[1], n3 = P.n[2];
-  for (int k = 0; k < M; ++k) {
-    GemmBatch b1;
-    b1.njobs = 0;
-    b1.total_tiles = 0;
-    int np = 0;
-    for (int q = 0; q < 3; ++q) {
-      const void* A[1] = {m + q * N};
-      const void* B[1] = {factor(&P, (const float*)T, k, q == 0 ? 1 : 0, 0)};
-      na_add(b1, np, n3 * n2, n1, n1, n3 * n2, Y + q * N, A, B, 1);
-    }
-    s = na_launch(&P, b1, st);
-    if (s != DEMAG_OK) return s;
-    GemmBatch b2;
-    b2.njobs = 0;
-    b2.total_tiles = 0;
-    np = 0;
-    const float* E2 = factor(&P, (const float*)T, k, 0, 1);
-    const float* F2 = factor(&P, (const float*)T, k, 1, 1);
-    {
-      const void* A[2] = {Y, Y + N};
-      const void* B[2] = {E2, F2};
-      na_add(b2, np, n1 * n3, n2, n2, n1 * n3, UV + (2 * k) * N, A, B, 2);
-    }
-    {
-      const void* A[1] = {Y + 2 * N};
-      const void* B[1] = {E2};
-      na_add(b2, np, n1 * n3, n2, n2, n1 * n3, UV + (2 * k + 1) * N, A, B, 1);
-    }
-    s = na_launch(&P, b2, st);
-    if (s != DEMAG_OK) return s;
-  }
-  GemmBatch b3;
-  b3.njobs = 0;
-  b3.total_tiles = 0;
-  int np = 0;
-  const void* A3[2 * kMaxTerms];
-  const void* B3[2 * kMaxTerms];
-  for (int k = 0; k < M; ++k) {
-    A3[2 * k] = UV + (2 * k) * N;
-    B3[2 * k] = factor(&P, (const float*)T, k, 0, 2);
-    A3[2 * k + 1] = UV + (2 * k + 1) * N;
-    B3[2 * k + 1] = factor(&P, (const float*)T, k, 1, 2);
-  }
-  na_add(b3, np, n2 * n1, n3, n3, n2 * n1, phi, A3, B3, 2 * M);
-  return na_launch(&P, b3, st);
+  // the mode-product chain of demag_apply_full (DEMAG_FP32), one node at a time
+  return mode_forward<float>(&P, m, phi, same_factors<float>(T), UV, Y, 1, 1.f, st);
 }
