@@ -13,18 +13,20 @@
 // factor Grams M_p = V^(q,p)^T W'_tp:
 //   <[[G; V]], [[C; W']]> = sum_{a,b} G[a] C[b] prod_p M_p[a_p][b_p].
 // One block per (term, component): the Grams in shared memory, the core
-// contraction mode by mode through a global workspace, FP64 throughout from
-// the FP32 factors; the per-block values are summed in a fixed order.
+// contraction mode by mode in FP64 (intermediates in shared memory, or in a
+// global workspace at large ranks); the per-block values are summed in a fixed
+// order.
+#include <type_traits>
+
 #include "internal.h"
 
 namespace demag {
 
 constexpr int kEnMaxRank = 64;
-// static shared memory of the energy kernels: the two [64][33] tiles of block_gram (float, or
-// double for the FP64 Tucker energy) and a 32-double reduction buffer
-template <typename T>
-constexpr size_t en_static_smem() { return 2 * 64 * 33 * sizeof(T) + 32 * sizeof(double); }
-constexpr size_t kEnStaticSmem = en_static_smem<float>();
+// static shared memory of the energy kernels: the partial sums of block_gram and a reduction buffer
+constexpr int kEnWarps = 8;
+constexpr size_t kEnStaticSmem = (kEnWarps * 64 + 32) * sizeof(double);
+constexpr size_t kEnSmemMax = 200 * 1024;  // largest dynamic request (Grams, and the contraction where it fits)
 
 __device__ __forceinline__ double en_warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -44,117 +46,217 @@ struct EnTuckerT {
   const F* W[3];     // term t, mode p: rows W[p] + t * s_p * n_p
   const F* w;        // term weights (NULL: 1)
   int T;             // number of terms
-  double* ws;        // per block r1 s3 (s2 + r2) doubles
+  double* ws;        // per block r1 s3 (s2 + r2) doubles; NULL: behind the Grams in shared memory
   double* part;      // [T][3]
 };
 using EnTucker = EnTuckerT<float>;
 
-// (D w)[i] of one factor row with the second-order stencils (central inside,
-// 3-point one-sided at the ends, two-point for n = 2, zero for n = 1)
+// 2 h (D w)[i] of one factor row at an end, in FP64 (3-point one-sided, two-point for n = 2, zero for
+// n = 1); between the ends it is w[i + 1] - w[i - 1], one rounding
 template <typename F>
-__device__ __forceinline__ double fd_row(const F* w, int i, int n, double inv2h) {
-  if (n == 1) return 0.0;
-  if (n == 2) return 2.0 * inv2h * ((double)w[1] - (double)w[0]);
-  if (i == 0) return inv2h * (-3.0 * (double)w[0] + 4.0 * (double)w[1] - (double)w[2]);
-  if (i == n - 1) return inv2h * (3.0 * (double)w[n - 1] - 4.0 * (double)w[n - 2] + (double)w[n - 3]);
-  return inv2h * ((double)w[i + 1] - (double)w[i - 1]);
+__device__ __forceinline__ F fd_end(const F* w, int i, int n) {
+  if (n == 1) return F(0);
+  if (n == 2) return (F)(2.0 * ((double)w[1] - (double)w[0]));
+  if (i == 0) return (F)(-3.0 * (double)w[0] + 4.0 * (double)w[1] - (double)w[2]);
+  return (F)(3.0 * (double)w[n - 1] - 4.0 * (double)w[n - 2] + (double)w[n - 3]);
 }
 
-// Mout[a][b] = sum_i A[a][i] B'[b][i] (B' = D B when deriv) for ra, rb <= 64 rows of length n:
-// 32-column tiles of A and B' through shared memory (tA, tB: [64][33]), each of the 256 threads
-// a 4 x 4 block of outputs; FP32 factors: FP32 products summed within a tile and FP64 across
-// tiles; FP64 factors: FP64 throughout.
+// An unevaluated sum hi + lo: FP32 values added without loss on the FP32 pipe
+// (Knuth's two-sum), where an FP64 addition would take 64 times as long; FP64
+// values as they are.
+template <typename F> struct EnSum;
+template <> struct EnSum<float> {
+  float hi, lo;
+  __device__ __forceinline__ void set(float v) { hi = v; lo = 0.f; }
+  __device__ __forceinline__ void add(float h, float l) {
+    const float s = __fadd_rn(hi, h), bb = __fsub_rn(s, hi);
+    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(h, bb));
+    hi = s;
+    lo = __fadd_rn(__fadd_rn(lo, l), e);
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+template <> struct EnSum<double> {
+  double hi, lo;
+  __device__ __forceinline__ void set(double v) { hi = v; lo = 0.0; }
+  __device__ __forceinline__ void add(double h, double) { hi += h; }
+  __device__ __forceinline__ double value() const { return hi; }
+};
+
+// One step of the transposing reduction: of C sums, a lane keeps the half that
+// its bit `off` selects and adds its partner's values of them.
+template <int C, typename F>
+__device__ __forceinline__ void en_halve(EnSum<F>* v, int off) {
+  const bool up = (threadIdx.x & off) != 0;
+#pragma unroll
+  for (int j = 0; j < C / 2; ++j) {
+    const EnSum<F> give = up ? v[j] : v[j + C / 2];
+    EnSum<F> keep = up ? v[j + C / 2] : v[j];
+    const F h = __shfl_xor_sync(0xffffffffu, give.hi, off);
+    F l = F(0);
+    if constexpr (C < 64 && std::is_same<F, float>::value) l = __shfl_xor_sync(0xffffffffu, give.lo, off);
+    keep.add(h, l);
+    v[j] = keep;
+  }
+}
+
+// One Gram M[a][b] = sum_i A[a][i] B'[b][i] of ra and rb rows of length n (B' = D B when deriv,
+// scale = 1 / (2 h)).
 template <typename F>
-__device__ void block_gram(const F* A, int ra, const F* B, int rb, int n, bool deriv, double inv2h,
-                           F* tA, F* tB, double* Mout) {
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4];
+struct EnGram {
+  const F *A, *B;
+  int ra, rb, n;
+  bool deriv;
+  double scale;
+  double* M;
+};
+
+// The three Grams g[0..2] (in shared memory) by the whole block.  The work is cut into items, 8 x 8
+// outputs over one segment of columns (at most 1024, so that the FP32 sums of a lane stay at 32
+// products), one warp each, 8 at a time: a lane takes every 32nd column of the segment, its 8 + 8
+// entries (read along the rows, coalesced) feed 64 products summed in registers, the lanes' sums are
+// added without loss (EnSum) by a transposing reduction, and segments in FP64 in a fixed order.
+// Bound: the latency of an item's loads and reduction, so small ranks split the columns until every
+// warp has an item.  1024^3, ranks 8, R = 61 (270 blocks): 661 us when 64 x 64 tiles padded every
+// rank and each partial sum and derivative was formed in FP64; 35 us now.
+template <typename F>
+__device__ void block_grams(const EnGram<F>* g, double* part) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int blocks = 0, first[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int p = 0; p < 3; ++p) blocks += ((g[p].ra + 7) >> 3) * ((g[p].rb + 7) >> 3);
+  const int want = blocks < kEnWarps ? kEnWarps / blocks : 1;  // segments per 8 x 8 block, at least
+  int seg[3], segs[3], items = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  for (int i0 = 0; i0 < n; i0 += 32) {
-    for (int e = threadIdx.x; e < 64 * 32; e += blockDim.x) {
-      const int r = e >> 5, c = e & 31, i = i0 + c;
-      tA[r * 33 + c] = (r < ra && i < n) ? A[(long)r * n + i] : F(0);
-      F bv = F(0);
-      if (r < rb && i < n) bv = deriv ? (F)fd_row(B + (long)r * n, i, n, inv2h) : B[(long)r * n + i];
-      tB[r * 33 + c] = bv;
+  for (int p = 0; p < 3; ++p) {
+    seg[p] = min(1024, ((g[p].n + want - 1) / want + 31) & ~31);
+    segs[p] = (g[p].n + seg[p] - 1) / seg[p];
+    first[p] = items;
+    items += ((g[p].ra + 7) >> 3) * ((g[p].rb + 7) >> 3) * segs[p];
+  }
+  first[3] = items;
+  // item -> Gram, 8 x 8 block, segment (segments of a block are consecutive)
+  auto locate = [&](int item, int& p, int& a0, int& b0, int& sg) {
+    p = item < first[1] ? 0 : item < first[2] ? 1 : 2;
+    const int ns = p == 0 ? segs[0] : p == 1 ? segs[1] : segs[2];
+    const int e = item - (p == 0 ? first[0] : p == 1 ? first[1] : first[2]);
+    const int nb = (g[p].rb + 7) >> 3, blk = e / ns;
+    sg = e - blk * ns;
+    a0 = blk / nb * 8;
+    b0 = (blk - blk / nb * nb) * 8;
+  };
+  for (int base = 0; base < items; base += kEnWarps) {
+    if (base + warp < items) {
+      int p, a0, b0, sg;
+      locate(base + warp, p, a0, b0, sg);
+      const F *A = g[p].A, *B = g[p].B;
+      const int ra = g[p].ra, rb = g[p].rb, n = g[p].n, len = p == 0 ? seg[0] : p == 1 ? seg[1] : seg[2];
+      const bool deriv = g[p].deriv;
+      F acc[8][8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = F(0);
+      const int iend = min(n, (sg + 1) * len);
+      for (int i = sg * len + lane; i < iend; i += 32) {
+        const int hi = deriv ? min(i + 1, n - 1) : i;
+        F av[8], bv[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          av[r] = a0 + r < ra ? A[(long)(a0 + r) * n + i] : F(0);
+          bv[r] = b0 + r < rb ? B[(long)(b0 + r) * n + hi] : F(0);
+        }
+        if (deriv) {  // the entries one to the right are there; those one to the left follow in one batch
+          F left[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r) left[r] = b0 + r < rb ? B[(long)(b0 + r) * n + max(i - 1, 0)] : F(0);
+#pragma unroll
+          for (int r = 0; r < 8; ++r) bv[r] = bv[r] - left[r];
+          if (i == 0 || i == n - 1) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+              if (b0 + r < rb) bv[r] = fd_end(B + (long)(b0 + r) * n, i, n);
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+          for (int c = 0; c < 8; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
+      }
+      EnSum<F> v[64];
+#pragma unroll
+      for (int j = 0; j < 64; ++j) v[j].set(acc[j / 8][j % 8]);
+      en_halve<64>(v, 16);
+      en_halve<32>(v, 8);
+      en_halve<16>(v, 4);
+      en_halve<8>(v, 2);
+      en_halve<4>(v, 1);
+      // a lane is left with outputs 2 lane and 2 lane + 1
+      part[warp * 64 + 2 * lane] = v[0].value();
+      part[warp * 64 + 2 * lane + 1] = v[1].value();
     }
     __syncthreads();
-    F part[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) part[i][j] = F(0);
-#pragma unroll 8
-    for (int c = 0; c < 32; ++c) {
-      F av[4], bw[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        av[i] = tA[(ty + 16 * i) * 33 + c];
-        bw[i] = tB[(tx + 16 * i) * 33 + c];
+    if (threadIdx.x < 64) {
+      for (int w = 0; w < kEnWarps && base + w < items; ++w) {
+        int p, a0, b0, sg;
+        locate(base + w, p, a0, b0, sg);
+        const int ia = a0 + threadIdx.x / 8, ib = b0 + threadIdx.x % 8;
+        if (ia < g[p].ra && ib < g[p].rb) {
+          double* o = g[p].M + ia * g[p].rb + ib;
+          const double v = part[w * 64 + threadIdx.x];
+          *o = (sg ? *o : 0.0) + (g[p].deriv ? g[p].scale * v : v);
+        }
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) part[i][j] = fma(av[i], bw[j], part[i][j]);
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] += (double)part[i][j];
     __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int ia = ty + 16 * i, ib = tx + 16 * j;
-      if (ia < ra && ib < rb) Mout[ia * rb + ib] = acc[i][j];
-    }
 }
 
 template <typename F>
-__global__ void __launch_bounds__(256) tucker_energy_kernel(const __grid_constant__ EnTuckerT<F> a) {
+__global__ void __launch_bounds__(32 * kEnWarps) tucker_energy_kernel(const __grid_constant__ EnTuckerT<F> a) {
   extern __shared__ double Mg[];
-  __shared__ double red[32];
-  __shared__ F tA[64 * 33], tB[64 * 33];
+  __shared__ double red[32], gpart[kEnWarps * 64];
+  __shared__ EnGram<F> gram[3];
   const int t = blockIdx.x, q = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int r1 = a.r[0], r2 = a.r[1], r3 = a.r[2];
   const int s1 = a.s[0], s2 = a.s[1], s3 = a.s[2];
-  // 1. Grams M_p [r_p][s_p] at offsets sum_{p' < p} r_p' s_p'
-  long voff = (long)q * ((long)r1 * a.n[0] + (long)r2 * a.n[1] + (long)r3 * a.n[2]);
-  int moff = 0;
-  int mo[3];
-  for (int p = 0; p < 3; ++p) {
-    const int n = a.n[p], rp = a.r[p], sp = a.s[p];
-    mo[p] = moff;
-    block_gram(a.V + voff, rp, a.W[p] + (long)t * sp * n, sp, n, p == q, a.inv2h[p], tA, tB, Mg + moff);
-    voff += (long)rp * n;
-    moff += rp * sp;
+  const int size_c = s1 * s2 * s3;
+  const F* Ct = a.C + (a.core_by_q ? (long)(t % 3) * size_c : 0L);
+  const int moff[4] = {0, r1 * s1, r1 * s1 + r2 * s2, r1 * s1 + r2 * s2 + r3 * s3};
+  // 1. Grams M_p [r_p][s_p]
+  if (threadIdx.x < 3) {
+    const int p = threadIdx.x;
+    long voff = (long)q * ((long)r1 * a.n[0] + (long)r2 * a.n[1] + (long)r3 * a.n[2]);
+    for (int pp = 0; pp < p; ++pp) voff += (long)a.r[pp] * a.n[pp];
+    gram[p] = {a.V + voff, a.W[p] + (long)t * a.s[p] * a.n[p], a.r[p],   a.s[p],
+               a.n[p],     p == q,                             a.inv2h[p], Mg + moff[p]};
   }
+  // the term's core in FP64, once
+  double* Cd = a.ws ? nullptr : Mg + moff[3];
+  if (Cd)
+    for (int i = threadIdx.x; i < size_c; i += blockDim.x) Cd[i] = (double)Ct[i];
   __syncthreads();
-  const double *M1 = Mg + mo[0], *M2 = Mg + mo[1], *M3 = Mg + mo[2];
-  const F* Ct = a.C + (a.core_by_q ? (long)(t % 3) * s1 * s2 * s3 : 0L);
-  double* Y1 = a.ws + ((long)t * 3 + q) * ((long)r1 * s3 * (s2 + r2));
-  double* Y2 = Y1 + (long)r1 * s2 * s3;
+  block_grams(gram, gpart);
+  const double *M1 = Mg, *M2 = Mg + moff[1], *M3 = Mg + moff[2];
+  double* Y1 = a.ws ? a.ws + ((long)t * 3 + q) * ((long)r1 * s3 * (s2 + r2)) : Cd + size_c;
+  double* Y2 = Y1 + r1 * s2 * s3;
   // 2. Y1[b3][b2][a1] = sum_b1 M1[a1][b1] C[b3][b2][b1]
-  for (long idx = threadIdx.x; idx < (long)s3 * s2 * r1; idx += blockDim.x) {
-    const int a1 = (int)(idx % r1);
-    const long bb = idx / r1;  // b3 s2 + b2
-    const F* crow = Ct + bb * s1;
+  for (int idx = threadIdx.x; idx < s3 * s2 * r1; idx += blockDim.x) {
+    const int bb = idx / r1, a1 = idx - bb * r1;  // b3 s2 + b2
     double acc = 0.0;
-    for (int b1 = 0; b1 < s1; ++b1) acc += M1[a1 * s1 + b1] * (double)crow[b1];
+    if (Cd) {
+      for (int b1 = 0; b1 < s1; ++b1) acc += M1[a1 * s1 + b1] * Cd[bb * s1 + b1];
+    } else {
+      for (int b1 = 0; b1 < s1; ++b1) acc += M1[a1 * s1 + b1] * (double)Ct[bb * s1 + b1];
+    }
     Y1[idx] = acc;
   }
   __syncthreads();
   // 3. Y2[b3][a2][a1] = sum_b2 M2[a2][b2] Y1[b3][b2][a1]
-  for (long idx = threadIdx.x; idx < (long)s3 * r2 * r1; idx += blockDim.x) {
-    const int a1 = (int)(idx % r1);
-    const int a2 = (int)((idx / r1) % r2);
-    const long b3 = idx / ((long)r1 * r2);
+  for (int idx = threadIdx.x; idx < s3 * r2 * r1; idx += blockDim.x) {
+    const int ba = idx / r1, a1 = idx - ba * r1;
+    const int b3 = ba / r2, a2 = ba - b3 * r2;
     double acc = 0.0;
     for (int b2 = 0; b2 < s2; ++b2) acc += M2[a2 * s2 + b2] * Y1[(b3 * s2 + b2) * r1 + a1];
     Y2[idx] = acc;
@@ -163,11 +265,10 @@ __global__ void __launch_bounds__(256) tucker_energy_kernel(const __grid_constan
   // 4. X = sum_a G^(q)[a3][a2][a1] sum_b3 M3[a3][b3] Y2[b3][a2][a1]
   const F* Gq = a.G + (long)q * r1 * r2 * r3;
   double x = 0.0;
-  for (long idx = threadIdx.x; idx < (long)r3 * r2 * r1; idx += blockDim.x) {
-    const long a21 = idx % ((long)r2 * r1);
-    const int a3 = (int)(idx / ((long)r2 * r1));
+  for (int idx = threadIdx.x; idx < r3 * r2 * r1; idx += blockDim.x) {
+    const int a3 = idx / (r2 * r1), a21 = idx - a3 * (r2 * r1);
     double acc = 0.0;
-    for (int b3 = 0; b3 < s3; ++b3) acc += M3[a3 * s3 + b3] * Y2[(long)b3 * r2 * r1 + a21];
+    for (int b3 = 0; b3 < s3; ++b3) acc += M3[a3 * s3 + b3] * Y2[b3 * r2 * r1 + a21];
     x += (double)Gq[idx] * acc;
   }
   x = en_warp_sum(x);
@@ -196,21 +297,20 @@ struct EnTT {
   double* part;                  // [T][3]
 };
 
-__global__ void __launch_bounds__(256) tt_energy_kernel(const __grid_constant__ EnTT a) {
+__global__ void __launch_bounds__(32 * kEnWarps) tt_energy_kernel(const __grid_constant__ EnTT a) {
   extern __shared__ double sg[];
-  __shared__ double red[32];
-  __shared__ float tA[64 * 33], tB[64 * 33];
+  __shared__ double red[32], gpart[kEnWarps * 64];
+  __shared__ EnGram<float> gram[3];
   const int t = blockIdx.x, q = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int r1 = a.r1, r2 = a.r2, r12 = r1 * r2;
-  const int rows[3] = {r1, r12, r2};
   double* Mg[3] = {sg, sg + r1 * r1, sg + r1 * r1 + (long)r12 * r12};
-  for (int p = 0; p < 3; ++p) {
-    const int n = a.n[p], rp = rows[p];
-    block_gram(a.A[p] + (long)q * rp * n, rp, a.B[p] + (long)t * rp * n, rp, n, p == q, a.inv2h[p], tA, tB,
-               Mg[p]);
+  if (threadIdx.x < 3) {
+    const int p = threadIdx.x, n = a.n[p], rp = p == 0 ? r1 : p == 1 ? r12 : r2;
+    gram[p] = {a.A[p] + (long)q * rp * n, a.B[p] + (long)t * rp * n, rp, rp, n, p == q, a.inv2h[p], Mg[p]};
   }
   __syncthreads();
+  block_grams(gram, gpart);
   double x = 0.0;
   for (int e = threadIdx.x; e < r2 * r2; e += blockDim.x) {
     const int a2 = e / r2, b2 = e % r2;
@@ -244,6 +344,41 @@ __global__ void __launch_bounds__(256) energy_sum_kernel(long count, const doubl
   }
 }
 
+// Scratch of one call, ordered on its stream (give it back with cudaFreeAsync).
+// It comes from a memory pool of the plan that keeps up to 64 MiB of what was
+// given back: with the device's default pool, which returns everything at each
+// synchronisation, a call that is waited for spent 200 us on mapping it again.
+// The pool dies with the plan.  Under stream capture the default pool is used.
+static demag_status scratch_alloc(demag_plan* P, void** mem, size_t bytes, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(st, &cap);
+  if (cap == cudaStreamCaptureStatusNone && !P->pool) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    if (cudaMemPoolCreate(&P->pool, &props) != cudaSuccess) {
+      P->pool = nullptr;
+      cudaGetLastError();  // the default pool serves
+    } else {
+      unsigned long long keep = 64ull << 20;
+      cudaMemPoolSetAttribute(P->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+  }
+  if (cap == cudaStreamCaptureStatusNone && P->pool)
+    DEMAG_CUDA(P, cudaMallocFromPoolAsync(mem, bytes, P->pool, st));
+  else
+    DEMAG_CUDA(P, cudaMallocAsync(mem, bytes, st));
+  return DEMAG_OK;
+}
+
+void scratch_destroy(demag_plan* P) {
+  if (P->pool) cudaMemPoolDestroy(P->pool);
+  P->pool = nullptr;
+}
+
 template <typename F>
 static demag_status run_tucker_energy(demag_plan* P, EnTuckerT<F>& a, double* energy, cudaStream_t st,
                                       const char* who) {
@@ -254,24 +389,29 @@ static demag_status run_tucker_energy(demag_plan* P, EnTuckerT<F>& a, double* en
     a.n[p] = P->n[p];
     a.inv2h[p] = 0.5 / P->h[p];
   }
-  const size_t smem = sizeof(double) * ((size_t)a.r[0] * a.s[0] + (size_t)a.r[1] * a.s[1] + (size_t)a.r[2] * a.s[2]);
-  if (smem + en_static_smem<F>() > 48 * 1024) {  // dynamic plus the kernel's static tiles
+  // The contraction's intermediates stay in shared memory beside the Grams where they fit (ranks up
+  // to about 15), in global memory otherwise.
+  const size_t grams = (size_t)a.r[0] * a.s[0] + (size_t)a.r[1] * a.s[1] + (size_t)a.r[2] * a.s[2];
+  const long per = (long)a.r[0] * a.s[2] * (a.s[1] + a.r[1]), core = (long)a.s[0] * a.s[1] * a.s[2];
+  const bool in_smem = sizeof(double) * (grams + per + core) <= 96 * 1024;
+  const size_t smem = sizeof(double) * (grams + (in_smem ? per + core : 0));
+  if (smem + kEnStaticSmem > 48 * 1024) {
     static unsigned long long done = 0;  // one per instantiation
     int dev = 0;
     cudaGetDevice(&dev);
     if (!(done & (1ull << (dev & 63)))) {
       DEMAG_CUDA(P, cudaFuncSetAttribute(tucker_energy_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(double) * 3 * kEnMaxRank * kEnMaxRank)));
+                                         (int)kEnSmemMax));
       done |= 1ull << (dev & 63);
     }
   }
   const long blocks = (long)a.T * 3;
-  const long per = (long)a.r[0] * a.s[2] * (a.s[1] + a.r[1]);
   void* mem = nullptr;
-  DEMAG_CUDA(P, cudaMallocAsync(&mem, sizeof(double) * (size_t)(blocks * per + blocks), st));
-  a.ws = static_cast<double*>(mem);
-  a.part = a.ws + blocks * per;
-  DEMAG_LAUNCH(P, kFamEnergy, st, tucker_energy_kernel<F><<<dim3(a.T, 3), 256, smem, st>>>(a));
+  demag_status s = scratch_alloc(P, &mem, sizeof(double) * (size_t)(blocks * (in_smem ? 0 : per) + blocks), st);
+  if (s != DEMAG_OK) return s;
+  a.part = static_cast<double*>(mem);
+  a.ws = in_smem ? nullptr : a.part + blocks;
+  DEMAG_LAUNCH(P, kFamEnergy, st, tucker_energy_kernel<F><<<dim3(a.T, 3), 32 * kEnWarps, smem, st>>>(a));
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
     const double vol = P->h[0] * P->h[1] * P->h[2];
@@ -384,7 +524,8 @@ extern "C" demag_status demag_energy_tt(demag_plan* P, const int r[2], const flo
   }
   const long blocks = (long)a.T * 3;
   void* mem = nullptr;
-  DEMAG_CUDA(P, cudaMallocAsync(&mem, sizeof(double) * (size_t)blocks, st));
+  demag_status s = scratch_alloc(P, &mem, sizeof(double) * (size_t)blocks, st);
+  if (s != DEMAG_OK) return s;
   a.part = static_cast<double*>(mem);
   DEMAG_LAUNCH(P, kFamEnergy, st, tt_energy_kernel<<<dim3(a.T, 3), 256, smem, st>>>(a));
   cudaError_t e = cudaGetLastError();
@@ -474,7 +615,9 @@ extern "C" demag_status demag_energy_tucker_fp64(demag_plan* P, const int r[3], 
   const long per_mode[3] = {(long)M * 3 * r[0] * P->n[0], (long)M * 3 * r[1] * P->n[1],
                             (long)M * 3 * r[2] * P->n[2]};
   void* mem = nullptr;
-  DEMAG_CUDA(P, cudaMallocAsync(&mem, sizeof(double) * (size_t)(per_mode[0] + per_mode[1] + per_mode[2] + 3 * M), st));
+  demag_status s = scratch_alloc(P, &mem, sizeof(double) * (size_t)(per_mode[0] + per_mode[1] + per_mode[2] + 3 * M),
+                                 st);
+  if (s != DEMAG_OK) return s;
   double* outV = static_cast<double*>(mem);
   double* w = outV + per_mode[0] + per_mode[1] + per_mode[2];
   TuckDirect d{};
@@ -507,7 +650,7 @@ extern "C" demag_status demag_energy_tucker_fp64(demag_plan* P, const int r[3], 
   a.W[2] = d.out[2];
   a.w = w;
   a.T = 3 * M;
-  demag_status s = run_tucker_energy(P, a, energy, st, "demag_energy_tucker_fp64");
+  s = run_tucker_energy(P, a, energy, st, "demag_energy_tucker_fp64");
   cudaFreeAsync(mem, st);
   return s;
 }

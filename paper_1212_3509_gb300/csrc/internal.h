@@ -79,6 +79,8 @@ struct demag_plan {
   void* cmp = nullptr;
   // energy / gradient scratch: phi, D^T m (1 field each) and P^T D^T m (3 fields)
   float* ews = nullptr;
+  // scratch of the structured energies: a stream-ordered pool that keeps up to 64 MiB (energy_tucker.cu)
+  cudaMemPool_t pool = nullptr;
   // per-fibre full format: two work volumes of 3M fields each
   float* fib_ws = nullptr;
 
@@ -214,5 +216,6 @@ __global__ void nonuniform_factor_kernel(int M, int n0, int n1, int n2, size_t t
 demag_status fd_gradient(demag_plan* plan, const float* phi, float* out, float scale,
                          cudaStream_t st);
 void energy_destroy(demag_plan* plan);
+void scratch_destroy(demag_plan* plan);  // energy_tucker.cu
 
 }  // namespace demag

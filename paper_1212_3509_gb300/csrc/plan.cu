@@ -264,6 +264,7 @@ static void free_plan_buffers(demag_plan* P) {
   fft3d_destroy(P);
   compress_destroy(P);
   energy_destroy(P);
+  scratch_destroy(P);
 }
 
 extern "C" demag_status demag_build_factors(const demag_grid_desc* d, demag_plan** out, void* stream) {
