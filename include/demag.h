@@ -500,13 +500,16 @@ demag_status demag_set_wait_limit(demag_plan* plan, double seconds);
  * layout.  enable = 0 runs the three-stage chain (each mode product's fields
  * in the workspace).  The adjoint (demag_apply_adjoint, its first two
  * transposed mode products fused the same way) and the analytic stray field
- * (demag_stray_field_exact) take the same schedule.  Both give the same values
+ * (demag_stray_field_exact) follow this call too.  Both give the same values
  * to rounding (the same
  * products, accumulated in another order); other grids and forms always run
- * the chain.  Without this call the plan takes the autotuner's choice
- * (demag_autotune, kind 9), else the fused schedule on grids of at least
- * 2^20 cells in the folded layout (about 100^3 and up) and the chain on
- * smaller ones.  Build-only; no counterpart in the paper. */
+ * the chain.  Without this call the forward application takes the autotuner's
+ * choice (demag_autotune, kind 9), else the fused schedule where ext1^2 ext2,
+ * the extents of the folded layout, is at least 4.5e6 (a cube of about 165^3;
+ * with fewer than 8 nodes, where the grid has 2^20 cells in that layout) and
+ * the chain elsewhere; the adjoint and the stray field take the fused one
+ * where ext1^2 ext2 is at least 1.2e7 (about 229^3).  Build-only; no
+ * counterpart in the paper. */
 demag_status demag_set_fused(demag_plan* plan, int enable);
 
 /* The forward schedule a plan's next full-format application in `prec`
@@ -599,7 +602,7 @@ demag_status demag_autotune(demag_plan* plan, int enable);
  * mode-3 stages of the fused forward and adjoint schedules), default value, 0;
  * schedule: 0, 1, 0, whatever the untuned choice), the chosen value, its time
  * per launch and the default value's time per launch in ms (for the schedule,
- * the untuned choice's time: fused from 2^20 folded cells, else the chain; 0
+ * the untuned choice's time, as under demag_set_fused; 0
  * for an entry read from a cache). */
 int demag_autotune_count(const demag_plan* plan);
 demag_status demag_autotune_entry(const demag_plan* plan, int i, int* kind, int key[3], int* value, float* ms,

@@ -8,14 +8,15 @@
 // product formed as A_hi B_hi + A_hi B_lo + A_lo B_hi with FP32 accumulation
 // in tensor memory.
 //
-// Kernel: persistent, one CTA (192 threads) per SM, warp-specialised:
+// Kernel: persistent, two CTAs (192 threads) per SM for tiles of up to 128
+// columns, one for wider ones, warp-specialised:
 //   warp 0      TMA producer: takes tiles from an atomic counter, hands their
 //               ids to the other roles through a shared ring, and loads
 //               A_hi, A_lo (128 rows) and B_hi, B_lo (BN rows) k-blocks of
-//               64-byte rows (32 BF16 or 16 TF32 elements) into a 4-stage
-//               shared-memory ring,
+//               64-byte rows (32 BF16 or 16 TF32 elements) into a
+//               shared-memory ring of as many stages as fit,
 //   warp 1      MMA issuer: 2 k-steps x 3 tcgen05.mma (M = 128, N = BN) per
-//               stage into one of two TMEM accumulators (2 x 256 columns),
+//               stage into one of two TMEM accumulators (128 or 256 columns each),
 //   warps 2..5  epilogue: tcgen05.ld of the accumulator (one TMEM lane per
 //               thread = one output row), then the hi/lo split of the next
 //               stage's operand or an FP32 field, stored transposed, through
@@ -77,6 +78,7 @@ constexpr int kOutStaging = kOutBufsPerWarp * kEpiWarps * kOutBuf;  // epilogue 
 // of 128 rows and B_hi, B_lo of the launch's widest N tile), staging, barriers
 constexpr int kSmemFixed = 1024 + kOutStaging + kBarBytes;
 constexpr int kSmemMax = 227 * 1024;
+constexpr int kSmemHalf = 113 * 1024;              // per CTA when two share an SM (1 KB each is reserved)
 constexpr int kTcThreads = 64 + 32 * kEpiWarps;
 constexpr int kRing = 4;                           // tile ids handed from the producer to the other roles
 // Every pipeline wait gives up after the plan's wait limit (default 2 s,
@@ -184,7 +186,10 @@ struct TcLaunch {
   int nstages;                         // operand stages in the ring (<= kMaxStages)
   int btile;                           // bytes of one B plane tile: widest N tile x 64
   int stage_bytes;                     // 2 kTileA + 2 btile
-  int* tile_counter;                   // zeroed before the launch
+  int acc_cols;                        // TMEM columns of one of the two accumulators (>= the widest N tile)
+  int* tile_counter;                   // zero before the launch
+  int* exits;                          // finished CTAs: the last one zeroes both for the next launch (NULL: the
+                                       // caller zeroes the tile counter)
   int* counters;                       // dependency counters, zeroed before the launch (or NULL)
   int* status;
   unsigned long long wait_ns;          // limit of every pipeline wait
@@ -233,6 +238,19 @@ __device__ __forceinline__ void epi_signal(int* counters, int ctr, int count, bo
     ptx::red_release_gpu_add(counters + ctr, count);
   }
   __syncwarp();
+}
+
+// A CTA that is done (every tile id it took is taken) counts itself; the last
+// one of the launch zeroes the work counter for the next launch, which saves a
+// memset before every launch.
+__device__ __forceinline__ void count_exit(int* work, int* exits) {
+  if (threadIdx.x == 0 && exits) {
+    __threadfence();
+    if (atomicAdd(exits, 1) == (int)gridDim.x - 1) {
+      *work = 0;
+      *exits = 0;
+    }
+  }
 }
 
 __device__ __forceinline__ void tc_fail(volatile int* abort, int* status) {
@@ -288,7 +306,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const __grid_con
     ptx::fence_mbar_init();
   }
   if (warp == 1) {
-    ptx::tmem_alloc(tmem_slot, 512);
+    ptx::tmem_alloc(tmem_slot, 2 * L.acc_cols);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
@@ -410,7 +428,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const __grid_con
           break;
         }
         ptx::tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(buf * kBN);
+        const uint32_t d = tmem_base + (uint32_t)(buf * L.acc_cols);
         uint32_t acc = 0;
         bool ok = true;
         for (int pi = 0; pi < J.npairs && ok; ++pi) {
@@ -491,13 +509,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const __grid_con
         epi_signal(L.counters, pend, pend_n, pend_tma, 0, lane);
         pend = -1;
       }
-      if (!ptx::mbar_wait(&tfull[buf], tph, abort, L.wait_ns)) {
+      // (a zero limit is taken at its word here, once per tile: the try of a bounded wait alone may
+      // block for longer than a short tile takes)
+      if (L.wait_ns == 0 ? !ptx::mbar_test_wait(&tfull[buf], tph)
+                         : !ptx::mbar_wait(&tfull[buf], tph, abort, L.wait_ns)) {
         tc_fail(abort, L.status);
         break;
       }
       ptx::tc_fence_after();
       int commits = 0;  // bulk groups lane 0 commits for this tile
-      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * kBN);
+      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * L.acc_cols);
       const int a0 = nt * G.bn;
       const int bn = G.bn;
       const int n_inner = G.n_inner;
@@ -691,7 +712,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const __grid_con
         if (armed & (1u << st)) ptx::mbar_wait(&full[st], (armed_par >> st) & 1u, &no_abort, kDrainNs);
     __syncthreads();
   }
-  if (warp == 1) ptx::tmem_dealloc(tmem_base, 512);
+  count_exit(L.tile_counter, L.exits);
+  if (warp == 1) ptx::tmem_dealloc(tmem_base, 2 * L.acc_cols);
 }
 
 // ---------------------------------------------------------------- fused mode-1 / mode-2 products
@@ -758,7 +780,8 @@ struct S12Launch {
   int kb1, kb2;                        // k-blocks of the two contractions (ceil(h1 / 32), ceil(h2 / 32))
   int pxor1, pxor2;                    // 1 when axis 1 / 2 carries derivative factors (dE odd, dF even)
   int units;                           // ext3 * M * 2 (batched: all items' units)
-  int* unit_counter;                   // zeroed before the launch
+  int* unit_counter;                   // zero before the launch
+  int* exits;                          // as in TcLaunch
   int* status;
   unsigned long long wait_ns;
   // batched launch (several grids, units numbered item after item): the
@@ -1262,6 +1285,7 @@ __global__ void __launch_bounds__(kS12Threads, 2) tc_s12_kernel(const __grid_con
         if (armed & (1u << st)) ptx::mbar_wait(&full[st], (armed_par >> st) & 1u, &no_abort, kDrainNs);
     __syncthreads();
   }
+  count_exit(L.unit_counter, L.exits);
   if (warp == 1) ptx::tmem_dealloc(tmem_base, kS12Tmem);
 }
 
@@ -1970,7 +1994,7 @@ struct TcState {
   void* buf1[2];          // [3M][ext1 ext3][ld2]
   void* buf2[2];          // [3M][ext2 ext1][ld3]
   int* status;
-  int* counter;           // dynamic tile counter of the running launch
+  int* counter;           // [2] dynamic tile counter of the running launch, its finished CTAs (both zero between launches)
   float* part;            // split node-sum partial fields
   int pp3;                // (A, B) pairs per accumulator in the node-sum stage
   int part_fields;        // partial fields allocated
@@ -1992,7 +2016,8 @@ struct TcState {
   // fields live in buf1
   bool fused;
   int sched;              // forward schedule (1 fused, 0 chain): the tuner's choice, else sched0
-  int sched0;             // untuned forward schedule: fused on grids of at least 2^20 split cells
+  int sched0;             // untuned forward schedule, by size
+  int sched_adj;          // schedule of the adjoint and the analytic stray field, by size
   S12Launch s12;
   S12Launch s12a;         // the adjoint's fused launch (Z with 3M fields)
   // analytic stray field: the forward stage programs with the derivative
@@ -2628,7 +2653,7 @@ demag_status tc_prepare(demag_plan* P, demag_precision prec, cudaStream_t st) {
     ok = ok && alloc(&S->buf2[h], 3 * (size_t)M * x2 * x1 * S->ld[2] * e);
   }
   ok = ok && alloc((void**)&S->status, sizeof(int));
-  ok = ok && alloc((void**)&S->counter, sizeof(int));
+  ok = ok && alloc((void**)&S->counter, 2 * sizeof(int));
   {
     const int kb3 = (geo.h[2] + kRowBytes / S->elem - 1) / (kRowBytes / S->elem);
     // TF32x3 issues twice the MMAs per K of BF16x3 in stages 1-2 as well, so its
@@ -2639,6 +2664,13 @@ demag_status tc_prepare(demag_plan* P, demag_precision prec, cudaStream_t st) {
     // which a grid of few rows needs (a batched application runs the same
     // stage on tensor cores, where more groups mean more tiles and partials)
     if (n3 <= kSmallAxis && x1 * x2 < 65536) S->pp3 = std::min(S->pp3, 4);
+    // on tensor cores likewise: a tile's pairs run one after another, so a grid
+    // of few rows gets more groups until every CTA slot has a tile (24^3 to 64^3:
+    // the node sum took 28 us whatever the size)
+    if (n3 > kSmallAxis) {
+      const long long tiles = (x1 * x2 + kBM - 1) / kBM * S->halves[2];
+      while (S->pp3 > 4 && tiles * ((2 * M + S->pp3 - 1) / S->pp3) < 304) S->pp3 = std::max(4, (S->pp3 + 1) / 2);
+    }
     const int gf = (2 * M + S->pp3 - 1) / S->pp3;   // forward: 2M pairs in one sum
     const int ga = (M + S->pp3 - 1) / S->pp3;       // adjoint: M pairs per component
     const int fields = gf > 3 * ga ? gf : 3 * ga;
@@ -2706,11 +2738,19 @@ demag_status tc_prepare(demag_plan* P, demag_precision prec, cudaStream_t st) {
     const int h1 = geo.h[0], h2 = geo.h[1], hq1 = geo.hq[0], hq2 = geo.hq[1];
     const int n2 = round_up(h2, 16);
     S->fused = S->elem == 2 && !P->nonuniform && geo.hq[0] && geo.hq[1] && geo.hq[2] && h1 <= 128 && h2 <= 128;
-    // untuned choice (BF16x3, R = 41, CUDA events per application): the chain
-    // is faster on small grids (32^3 0.072 against 0.095 ms, 80^3 0.249 against
-    // 0.274, 96^3 0.325 against 0.329), the fused schedule from 112^3 on
-    // (0.42 against 0.45 ms, 160^3 0.87 against 0.99, 256^3 2.14 against 3.00)
-    S->sched0 = x1 * x2 * x3 >= (1LL << 20) ? 1 : 0;
+    // Untuned choice.  The fused kernel's unit is a slab and a node whatever h1 is (its A tile has 128
+    // rows), and its hand-offs are paid per chunk of h2 columns, so what it does per unit of time grows
+    // with ext1 and with ext1 ext2, while the chain's time follows the cells: the line is drawn at
+    // ext1^2 ext2.  BF16x3, R = 41, chain against fused, us: 128^3 385 / 418, 160^3 760 / 819,
+    // 176^3 1214 / 1154, 256^3 2761 / 2108, 53 x 204 x 181 692 / 1040, 256 x 128 x 128 697 / 606,
+    // 128 x 256 x 256 1447 / 1588 (41 grids, each also at R = 11, 21, 61: the same side but for ties).
+    // With fewer than 8 nodes the two differ by 10 us or so on the grids between; those keep the
+    // line at 2^20 split cells.
+    S->sched0 = x1 * x1 * x2 >= 4500000LL || (M < 8 && x1 * x2 * x3 >= (1LL << 20)) ? 1 : 0;
+    // The adjoint (three targets per unit instead of two, mode-1 tiles formed twice) and the stray
+    // field (one fused launch per direction where the chain shares stages): 192^3 1192 / 1200 and
+    // 3064 / 3043, 224^3 2171 / 2198, 240 x 208 x 66 1042 / 981, 256^3 2751 / 2569 and 7046 / 6189.
+    S->sched_adj = x1 * x1 * x2 >= 12000000LL ? 1 : 0;
     S->sched = S->sched0;
     if (S->fused) {
       S12Launch& Z = S->s12;
@@ -2789,7 +2829,14 @@ static demag_status launch_segs(demag_plan* P, const TcGroup* groups, const TcSe
   // as many operand stages of the launch's widest N tile as fit
   L.btile = maxbn * kRowBytes;
   L.stage_bytes = (2 * kTileA + 2 * L.btile + 1023) / 1024 * 1024;
-  L.nstages = std::min(kMaxStages, (kSmemMax - kSmemFixed) / L.stage_bytes);
+  // Tiles of at most 128 columns: two CTAs per SM, each with half the tensor memory and shared memory.
+  // A tile's life (fill, a short MMA run, the drain of its accumulator through four warps) leaves most
+  // of an SM's units idle most of the time, and the CTAs fill each other's gaps.  R = 41, one against
+  // two CTAs: BF16x3 chain 64^3 135 -> 105 us, 128^3 518 -> 386, 256^3 2999 -> 2758 (its node sum after
+  // the fused kernel 563 -> 532); TF32x3 96^3 457 -> 337, 192^3 2647 -> 2319.
+  const bool two = maxbn <= 128;
+  L.acc_cols = two ? 128 : kBN;
+  L.nstages = std::min(kMaxStages, ((two ? kSmemHalf : kSmemMax) - kSmemFixed) / L.stage_bytes);
   if (want_stages > 0) L.nstages = std::min(L.nstages, want_stages);
   const int smem_bytes = kSmemFixed + L.nstages * L.stage_bytes;
   L.tile_counter = counter;
@@ -2799,9 +2846,12 @@ static demag_status launch_segs(demag_plan* P, const TcGroup* groups, const TcSe
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = total_tiles < sms ? total_tiles : sms;
-  // the dependency counters follow the tile counter in the same buffer when present
-  DEMAG_CUDA(P, cudaMemsetAsync(counter, 0, sizeof(int) * (1 + (counters ? ncounters : 0)), st));
+  const int most = two ? 2 * sms : sms;
+  const int grid = total_tiles < most ? total_tiles : most;
+  // a launch with dependency counters (they follow the tile counter in the same buffer) needs them all
+  // zeroed; without, the previous launch left the tile counter at zero
+  L.exits = counters ? nullptr : counter + 1;
+  if (counters) DEMAG_CUDA(P, cudaMemsetAsync(counter, 0, sizeof(int) * (1 + ncounters), st));
   DEMAG_LAUNCH(P, kFamGemmTc, st, tc_gemm_kernel<F><<<grid, kTcThreads, smem_bytes, st>>>(L));
   DEMAG_LAUNCHED(P, "tc_gemm_kernel");
   return DEMAG_OK;
@@ -2969,7 +3019,7 @@ static demag_status run_s12(demag_plan* P, TcState* S, const S12Launch& base, cu
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = L.units < 2 * sms ? L.units : 2 * sms;  // two CTAs per SM
-  DEMAG_CUDA(P, cudaMemsetAsync(S->counter, 0, sizeof(int), st));
+  L.exits = S->counter + 1;
   if (adj)
     DEMAG_LAUNCH(P, kFamGemmTc, st, tc_s12_kernel<true, false><<<grid, kS12Threads, kS12Smem, st>>>(L));
   else
@@ -2994,8 +3044,8 @@ static demag_status forward_chain(demag_plan* P, TcState* S, const float* m, flo
 template <class F>
 static demag_status adjoint_chain(demag_plan* P, TcState* S, const float* y, float* g, cudaStream_t st) {
   demag_status s = split_input<F>(P, S, y, 1, st);
-  if (S->fused && (P->fused > 0 || (P->fused < 0 && S->sched))) {
-    // the forward's schedule: the first two transposed mode products fused
+  if (S->fused && (P->fused > 0 || (P->fused < 0 && S->sched_adj))) {
+    // the first two transposed mode products fused
     if (s == DEMAG_OK) s = run_s12(P, S, S->s12a, st, true);
     if (s == DEMAG_OK) s = run_program<F>(P, S, kAdj3Z, st);
     if (s != DEMAG_OK) return s;
@@ -3098,13 +3148,43 @@ demag_status tc_batch_create(demag_plan* const* plans, int count, demag_precisio
       ++SB.count;
     }
   }
+  // Tiles wider than 128 columns (an axis half above 128: long films, non-uniform grids) would hold
+  // the whole launch to one CTA per SM (launch_segs).  Where they carry less than half of its output
+  // they are cut into equal ones of at most 128: 16 uneven grids with two 512 x 512 x 4 films 7.20 ms
+  // uncut, 6.36 cut.  Alone, such grids are faster with the wide tiles (512 x 512 x 4 434 against
+  // 453 us, 256^3 non-uniform 3.28 against 3.97 ms), which keep their A operand's rows longer.
+  {
+    double wide = 0, all = 0;
+    for (const TcGroup& gg : g) {
+      const double w = (double)gg.njobs * gg.rows * gg.n_a;
+      all += w;
+      if (gg.bn > 128) wide += w;
+    }
+    if (wide > 0 && wide < 0.5 * all)
+      for (int i = 0; i < count; ++i)
+        for (int st3 = 0; st3 < 3; ++st3) {
+          TcGroup& G = g[st3 * count + i];
+          if (G.bn <= 128) continue;
+          const TcState* S = state(plans[order[i]], prec);
+          const int axis = B->fused[order[i]] && st3 == 0 ? 2 : st3;
+          const int tiles = (G.n_a + 127) / 128;
+          G.bn = round_up((G.n_a + tiles - 1) / tiles, 16);
+          G.n_tiles = (G.n_a + G.bn - 1) / G.bn;
+          G.ntiles = G.njobs * G.m_tiles * G.n_tiles;
+          for (int h = 0; h < 2; ++h)
+            if (!make_bmap(h ? &G.b_lo : &G.b_hi, S->B[axis][h], S->elem, S->geo.h[axis], S->halves[axis],
+                           2 * plans[order[i]]->M, S->ldB[axis], G.bn)) {
+              tc_batch_destroy(B);
+              return set_error(P0, DEMAG_ECUDA, "tensor map encoding failed");
+            }
+        }
+  }
   int acc = 0;
   // passes: chain stage 1, fused mode-3 stages, chain stages 2 and 3
   for (int pass = 0; pass < 4; ++pass) {
     for (int i = 0; i < count; ++i) {
       const bool fz = B->fused[order[i]] != 0;
       if (fz != (pass == 1)) continue;
-      const TcState* S = state(plans[order[i]], prec);
       const int st3 = pass == 0 ? 0 : pass - 1;
       if (st3 == 2 && thin3[i]) continue;  // in the CUDA-core launch after this one
       const int gi = fz ? i : st3 * count + i;
@@ -3112,7 +3192,7 @@ demag_status tc_batch_create(demag_plan* const* plans, int count, demag_precisio
       TcSeg q = whole_seg(g[gi], gi, acc);
       if (!fz && st3 > 0) {
         q.dep = 2 * i + (st3 - 1);
-        q.dep_target = kEpiWarps * S->host_prog[kFwd1 + st3 - 1].ntiles;
+        q.dep_target = kEpiWarps * g[(st3 - 1) * count + i].ntiles;
       }
       if (!fz && st3 < 2) q.done = 2 * i + st3;
       segs.push_back(q);
@@ -3316,7 +3396,7 @@ static demag_status field_chain(demag_plan* P, TcState* S, const float* m, float
   const long long N = (long long)P->n[0] * P->n[1] * P->n[2];
   demag_status s = prepare_field<F>(P, S, st);
   if (s == DEMAG_OK) s = split_input<F>(P, S, m, 3, st);
-  if (S->fused && (P->fused > 0 || (P->fused < 0 && S->sched))) {
+  if (S->fused && (P->fused > 0 || (P->fused < 0 && S->sched_adj))) {
     // the fused schedule, once per direction (the stage-1 fields are never
     // stored, so the directions share nothing but the split input): direction
     // 3 the fused launch and the derivative mode-3 stage, directions 2 and 1
