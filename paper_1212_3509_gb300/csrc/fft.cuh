@@ -136,6 +136,218 @@ __device__ __forceinline__ void dft_reg(C (&v)[R]) {
   }
 }
 
+// The first 8 outputs of an inverse 16-point DFT (the kept half of the last
+// pass): two 8-point DFTs of the even and odd inputs and the "+" half of the
+// final butterflies.
+template <int K>
+__device__ __forceinline__ void combine_half16(float2 (&v)[16], float2 (&e)[8], float2 (&o)[8]) {
+  if constexpr (K < 8) {
+    const float2 t = rot<16, K, true>(o[K]);
+    if constexpr (K == 4) {  // +i: folded into scalar adds
+      v[K].x = e[K].x + t.x;
+      v[K].y = e[K].y + t.y;
+    } else {
+      v[K] = cadd(e[K], t);
+    }
+    combine_half16<K + 1>(v, e, o);
+  }
+}
+
+__device__ __forceinline__ void idft16_first_half(float2 (&v)[16]) {
+  float2 e[8], o[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    e[i] = v[2 * i];
+    o[i] = v[2 * i + 1];
+  }
+  dft_reg<8, true>(e);
+  dft_reg<8, true>(o);
+  combine_half16<0>(v, e, o);
+}
+
+// v[r] *= exp(-2 pi i r / 16), r < 8
+template <int R>
+__device__ __forceinline__ void rot16_rows(float2 (&v)[8]) {
+  if constexpr (R < 8) {
+    v[R] = rot<16, R, false>(v[R]);
+    rot16_rows<R + 1>(v);
+  }
+}
+
+// Forward 16-point DFT of inputs r < 8 (the others are zero): the even outputs
+// are the 8-point DFT of the inputs, the odd ones that of x_r W_16^r.
+__device__ __forceinline__ void dft16_of_half(const float2 (&x)[8], float2 (&v)[16]) {
+  float2 e[8], o[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) e[r] = o[r] = x[r];
+  rot16_rows<1>(o);
+  dft_reg<8, false>(e);
+  dft_reg<8, false>(o);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    v[2 * m] = e[m];
+    v[2 * m + 1] = o[m];
+  }
+}
+
+// ---- FFT of length N = 16 B, 32 <= N <= 512, in the registers of B lanes ----
+//
+// Lane l (of the B consecutive lanes of a fibre) holds 16 elements.  In time
+// order element r is x[l + B r]; in frequency order element s is X[f(l, s)]
+// (rf_freq), a fixed permutation that a product with a spectrum does not mind.
+// With f = k1 + 16 k2, X = sum_j W_B^(j k2) [ W_N^(j k1) sum_r W_16^(r k1) x[j + B r] ]:
+// a 16-point DFT in registers, one twiddle, one exchange through shared memory
+// (16 rows of B, one write and one read of the fibre), and 16 / B DFTs of B
+// points in registers; for B = 32 a 32-point one shared by two lanes, its last
+// radix-2 step by shuffles.  The inverse takes the same steps backwards.  A
+// fibre thus crosses shared memory once per transform where the in-place
+// radix-16 passes of fft_inplace cross it once per pass and once to be staged.
+// Only the first N / 2 time samples exist (zero padding in, kept half out).
+//
+// Exchange rows are B + 1 long and a fibre's buffer is N + 17 long (1 mod 16):
+// with fibre g in slot rf_slot(g) the fibres that share a half-warp lie B
+// apart modulo 16, so rows, columns and (16 fibres of one index) transposed
+// reads are all free of bank conflicts.
+template <int B> struct RegFft {
+  static constexpr int N = 16 * B;
+  static constexpr int BS = N + 17;  // buffer elements per fibre
+};
+
+template <int B>
+__device__ __forceinline__ int rf_slot(int g) {
+  if constexpr (B >= 16) return g;
+  constexpr int F = B >= 16 ? 1 : 16 / B;  // fibres per half-warp
+  return (g & ~15) + (g % F) * B + (g / F) % B;
+}
+
+template <int B>
+__device__ __forceinline__ int rf_freq(int l, int s) {
+  if constexpr (B == 32) return (l & 15) + 16 * (8 * (l >> 4) + (s & 7) + 16 * (s >> 3));
+  return l + B * (s / B) + 16 * (s % B);
+}
+
+__device__ __forceinline__ float2 shfl_xor2(float2 v, int off) {
+  v.x = __shfl_xor_sync(0xffffffffu, v.x, off);
+  v.y = __shfl_xor_sync(0xffffffffu, v.y, off);
+  return v;
+}
+
+// exp(-2 pi i t / 32), t < 8
+__device__ __forceinline__ constexpr double w32_re(int t) {
+  return t == 0 ? 1.0 : t == 1 ? 0.98078528040323044913 : t == 2 ? 0.92387953251128675613
+       : t == 3 ? 0.83146961230254523708 : t == 4 ? 0.70710678118654752440 : t == 5 ? 0.55557023301960222474
+       : t == 6 ? 0.38268343236508977173 : 0.19509032201612826785;
+}
+__device__ __forceinline__ constexpr double w32_im(int t) { return t == 0 ? 0.0 : -w32_re(8 - t); }
+
+template <bool INV, int T>
+__device__ __forceinline__ float2 rot32(float2 v) {
+  float2 w;
+  w.x = (float)w32_re(T);
+  w.y = INV ? -(float)w32_im(T) : (float)w32_im(T);
+  return T == 0 ? v : cmul(v, w);
+}
+
+// The radix-2 step of B = 32 for t = T..7: forward on (B_0, B_1)[k2'], k2' = 8 h + t
+template <int T>
+__device__ __forceinline__ void rf_join(float2 (&u)[16], const float2 (&other)[8], int h) {
+  if constexpr (T < 8) {
+    const float2 own = h ? u[8 + T] : u[T];
+    const float2 b0 = h ? other[T] : own;
+    float2 c = rot32<false, T>(h ? own : other[T]);
+    if (h) c = make_float2(c.y, -c.x);  // W_32^(8 + t) = -i W_32^t
+    rf_join<T + 1>(u, other, h);        // (reads u[T + 1 ..], u[8 + T + 1 ..] before they are written)
+    u[T] = cadd(b0, c);
+    u[8 + T] = csub(b0, c);
+  }
+}
+template <int T>
+__device__ __forceinline__ void rf_part(float2 (&u)[16], float2 (&send)[8], float2 (&keep)[8], int h) {
+  if constexpr (T < 8) {
+    const float2 b = cadd(u[T], u[8 + T]);
+    float2 c = rot32<true, T>(csub(u[T], u[8 + T]));
+    if (h) c = make_float2(-c.y, c.x);  // conj W_32^(8 + t) = i conj W_32^t
+    send[T] = h ? b : c;
+    keep[T] = h ? c : b;
+    rf_part<T + 1>(u, send, keep, h);
+  }
+}
+
+// x: the 8 time samples x[l + B r]; u: the spectrum in frequency order.  pw[r] = W_N^(l r).
+template <int B>
+__device__ __forceinline__ void rf_forward(const float2 (&x)[8], float2 (&u)[16], float2* buf, int l,
+                                           const float2 (&pw)[16]) {
+  {
+    float2 v[16];
+    dft16_of_half(x, v);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) buf[k * (B + 1) + l] = k ? cmul(v[k], pw[k]) : v[k];
+  }
+  __syncwarp();
+  if constexpr (B == 32) {
+    const int k1 = l & 15, h = l >> 4;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) u[i] = buf[k1 * (B + 1) + 2 * i + h];
+    __syncwarp();
+    dft_reg<16, false>(u);
+    float2 other[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) other[t] = shfl_xor2(h ? u[t] : u[8 + t], 16);
+    rf_join<0>(u, other, h);
+  } else {
+    constexpr int E = B >= 16 ? 1 : 16 / B;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      float2 w[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) w[j] = buf[(l + B * e) * (B + 1) + j];
+      dft_reg<B, false>(w);
+#pragma unroll
+      for (int j = 0; j < B; ++j) u[e * B + j] = w[j];
+    }
+    __syncwarp();
+  }
+}
+
+// u: a spectrum in frequency order; v[r], r < 8: x[l + B r] of the unnormalised inverse.
+template <int B>
+__device__ __forceinline__ void rf_inverse(float2 (&u)[16], float2 (&v)[16], float2* buf, int l,
+                                           const float2 (&pw)[16]) {
+  if constexpr (B == 32) {
+    const int k1 = l & 15, h = l >> 4;
+    float2 send[8], keep[8];
+    rf_part<0>(u, send, keep, h);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const float2 got = shfl_xor2(send[t], 16);
+      u[t] = h ? got : keep[t];
+      u[8 + t] = h ? keep[t] : got;
+    }
+    dft_reg<16, true>(u);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) buf[k1 * (B + 1) + 2 * i + h] = u[i];
+  } else {
+    constexpr int E = B >= 16 ? 1 : 16 / B;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      float2 w[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) w[j] = u[e * B + j];
+      dft_reg<B, true>(w);
+#pragma unroll
+      for (int j = 0; j < B; ++j) buf[(l + B * e) * (B + 1) + j] = w[j];
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float2 y = buf[k * (B + 1) + l];
+    v[k] = k ? cmul(y, make_float2(pw[k].x, -pw[k].y)) : y;
+  }
+  __syncwarp();
+  idft16_first_half(v);
+}
+
 // Radix plan for N = 2^LOGN: number of radix-16 passes and the remainder radix.
 template <int LOGN> struct RadixPlan {
   static constexpr int n16 = LOGN / 4;

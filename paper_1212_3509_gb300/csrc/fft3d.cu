@@ -42,6 +42,8 @@ namespace demag {
 
 constexpr int kFft3dMaxLog = 11;  // L_p <= 2048 (n_p <= 1024)
 
+// Lengths 32 to 512 run in registers (R3 below); shorter and longer ones by
+// in-place passes in shared memory, this way:
 // Launch shape for an FFT of length N = 2^LOGN along one axis: TG threads
 // per fibre, G fibres per block (at least 16, so that the transposed stores
 // write runs of >= 128 bytes), buffers padded by pad16 and separated by an
@@ -52,8 +54,8 @@ constexpr int kFft3dMaxLog = 11;  // L_p <= 2048 (n_p <= 1024)
 constexpr int f3_tg(int N) { return N >= 2048 ? 128 : (N / 16 < 1 ? 1 : (N / 16 > 32 ? 32 : N / 16)); }
 constexpr int f3_fibres(int N) { return N >= 2048 ? 4 : (16 * f3_tg(N) < 256 ? 256 / f3_tg(N) : 16); }
 constexpr int f3_block(int N) { return f3_fibres(N) * f3_tg(N); }
-// P3 double-buffers its fibres: half the fibres per block for N = 512 and
-// 1024 (two blocks of 256 threads per SM at 128 registers instead of one of
+// P3 holds more per fibre: half the fibres per block for N = 512 and 1024
+// (two blocks of 256 threads per SM at 128 registers instead of one of
 // 512); N = 2048 keeps its 4 fibres (512 threads, one block per SM)
 constexpr int f3_fibres_p3(int N) {
   return N >= 2048 ? f3_fibres(N) : (N >= 512 ? f3_fibres(N) / 2 : f3_fibres(N));
@@ -73,10 +75,6 @@ template <int LOGN> struct F3 {
   static constexpr size_t smem3 = ((size_t)N + (size_t)2 * G3 * BS) * sizeof(float2);
   static constexpr size_t smem3f = ((size_t)N + (size_t)3 * G3 * BS) * sizeof(float2);  // field: 3 spectra
   static constexpr int PER = N / TG;  // bins per thread of its fibre
-  // N = 2^(4j+1): the radix-2 pass is skipped on zero-padded input (forward)
-  // and folded into the reader of the first N/2 outputs (inverse)
-  static constexpr bool FOLD = LOGN >= 5 && LOGN % 4 == 1;
-  static constexpr int SL = FOLD ? N / 2 : N;  // staged length of a forward input
 };
 
 // Synchronise the threads of one FFT group: a warp when the group lies inside
@@ -163,104 +161,6 @@ __device__ __forceinline__ void fft_pad(float2* buf, int lt, const float2* tw) {
   }
 }
 
-// One in-place radix-16 Stockham pass over sub-transforms of size Ns.  With
-// DUP the pass input is y[m] = x[m >> 1]: the output of a radix-2 first pass
-// on an input with x[j] = 0 for j >= N/2, which only duplicates
-// (y[2j] = y[2j+1] = x[j]) and is therefore not done.
-template <int LOGN, bool INV, bool DUP>
-__device__ __forceinline__ void r16_pass(float2* buf, int Ns, int lt, const float2* tw) {
-  using C = F3<LOGN>;
-  constexpr int N = C::N, TG = C::TG;
-  constexpr int items = N / 16;
-  constexpr int ipt = (items + TG - 1) / TG;
-  float2 v[ipt][16];
-#pragma unroll
-  for (int it = 0; it < ipt; ++it) {
-    const int j = lt + it * TG;
-    if (items % TG == 0 || j < items) {
-      const int k = j % Ns;
-#pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        // pad16(i + r S) = pad16(i) + r (S + S/16) when S is a multiple of 16
-        if constexpr (DUP && (items / 2) % 16 == 0)
-          v[it][r] = buf[pad16(j >> 1) + r * PadStride<items / 2>::value];
-        else if constexpr (!DUP && items % 16 == 0)
-          v[it][r] = buf[pad16(j) + r * PadStride<items>::value];
-        else
-          v[it][r] = buf[pad16(DUP ? ((j + r * items) >> 1) : (j + r * items))];
-      }
-      if (Ns > 1) {  // (Ns = 1: all twiddles are 1)
-        float2 w = tw[k * (N / (Ns * 16))];
-        if (INV) w.y = -w.y;
-        float2 pw[16];
-        powers<16>(w, pw);
-#pragma unroll
-        for (int r = 1; r < 16; ++r) v[it][r] = cmul(v[it][r], pw[r]);
-      }
-      dft_reg<16, INV>(v[it]);
-    }
-  }
-  group_sync<TG>();
-#pragma unroll
-  for (int it = 0; it < ipt; ++it) {
-    const int j = lt + it * TG;
-    if (items % TG == 0 || j < items) {
-      const int k = j % Ns;
-      const int base = (j / Ns) * Ns * 16 + k;
-      if (Ns % 16 == 0) {
-        const int b0 = pad16(base), step = Ns + (Ns >> 4);
-#pragma unroll
-        for (int r = 0; r < 16; ++r) buf[b0 + r * step] = v[it][r];
-      } else {
-#pragma unroll
-        for (int r = 0; r < 16; ++r) buf[pad16(base + r * Ns)] = v[it][r];
-      }
-    }
-  }
-  group_sync<TG>();
-}
-
-// Forward FFT of a fibre staged in its first SL slots (zeros past the data).
-template <int LOGN>
-__device__ __forceinline__ void fwd_fft(float2* buf, int lt, const float2* tw) {
-  using C = F3<LOGN>;
-  if constexpr (C::FOLD) {
-    r16_pass<LOGN, false, true>(buf, 2, lt, tw);
-#pragma unroll
-    for (int ps = 2, Ns = 32; ps < C::NPASS; ++ps, Ns *= 16) r16_pass<LOGN, false, false>(buf, Ns, lt, tw);
-  } else {
-    fft_pad<LOGN, false>(buf, lt, tw);
-  }
-}
-
-// Inverse FFT whose outputs k < N/2 are then read with inv_out (with FOLD the
-// last radix-2 pass is left to inv_out).
-template <int LOGN>
-__device__ __forceinline__ void inv_fft(float2* buf, int lt, const float2* tw) {
-  using C = F3<LOGN>;
-  if constexpr (C::FOLD) {
-#pragma unroll
-    for (int ps = 1, Ns = 1; ps < C::NPASS; ++ps, Ns *= 16) r16_pass<LOGN, true, false>(buf, Ns, lt, tw);
-  } else {
-    fft_pad<LOGN, true>(buf, lt, tw);
-  }
-}
-
-// Output k < N/2 of inv_fft: with FOLD the last radix-2 butterfly (Ns = N/2)
-// y_k = x_k + conj(W_N^k) x_{k + N/2}.
-template <int LOGN>
-__device__ __forceinline__ float2 inv_out(const float2* buf, int k, const float2* tw) {
-  using C = F3<LOGN>;
-  if constexpr (C::FOLD) {
-    float2 w = tw[k];
-    w.y = -w.y;
-    const float2 a = buf[pad16(k)], b = buf[pad16(k + C::N / 2)];
-    return cadd(a, cmul(b, w));
-  } else {
-    return buf[pad16(k)];
-  }
-}
-
 struct Fft3dArgs {
   int n1, n2, n3;
   int L1, L2, L3;
@@ -271,7 +171,7 @@ struct Fft3dArgs {
   float* phi;             // [n3][n2][n1]
   const float* kst;       // [3][H1][H2][H3]: Im K^(q) on the octant
   const float* kfield;    // [6][H1][H2][H3]: the real field kernels K_pq on the octant (pairs 00 11 22 01 02 12)
-  const float2* tw;       // exp(-2 pi i m / N) of this pass's axis, m < N
+  const float2* tw;       // this pass's axis: exp(-2 pi i m / N), m < N, or the table of rf_twiddles
   int nco;                // components after P3: 1 (potential) or 3 (field)
 };
 
@@ -341,7 +241,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p1_kernel(const __grid_
   const float* row = a.m + (size_t)ci3 * a.n2 * a.n1;
   const bool va = i2a < a.n2, vb = i2a + 1 < a.n2;
   // all loads of the fibre pair in flight before the first shared-memory store
-  constexpr int CNT = C::SL / TG;
+  constexpr int CNT = N / TG;
   float2 ld[CNT];
 #pragma unroll
   for (int i = 0; i < CNT; ++i) {
@@ -356,7 +256,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p1_kernel(const __grid_
 #pragma unroll
   for (int i = 0; i < CNT; ++i) buf[pad16(lt + i * TG)] = ld[i];
   __syncthreads();
-  fwd_fft<LOGN>(buf, lt, tw);
+  fft_pad<LOGN, false>(buf, lt, tw);
   __syncthreads();  // the split step reads every fibre pair's buffer
   // X_a = (Z_w + conj Z_{N-w}) / 2, X_b = (Z_w - conj Z_{N-w}) / 2i; stored at S1[c][w][i3][i2]
   const int c = ci3 / a.n3, i3 = ci3 % a.n3;
@@ -402,9 +302,9 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p2_kernel(const __grid_
   const int cw1 = blockIdx.x / tiles;  // c * H1 + w1
   const int i3 = tile * G + g;
   const float2* in = a.s1 + ((size_t)cw1 * a.n3 + i3) * a.n2;
-  stage_fibre<LOGN, C::SL>(buf, lt, in, i3 < a.n3 ? a.n2 : 0);
+  stage_fibre<LOGN, C::N>(buf, lt, in, i3 < a.n3 ? a.n2 : 0);
   __syncthreads();
-  fwd_fft<LOGN>(buf, lt, tw);
+  fft_pad<LOGN, false>(buf, lt, tw);
   __syncthreads();  // the transposed store reads every fibre's buffer
   const int c = cw1 / a.H1, w1 = cw1 % a.H1;
   float2* out = a.s2 + (size_t)c * a.L2 * a.H1 * a.n3 + (size_t)w1 * a.n3 + (size_t)tile * G;
@@ -440,7 +340,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3_
   const int w2f = w2 <= a.L2 / 2 ? w2 : a.L2 - w2;
   const int nload = valid ? a.n3 : 0;
   auto fibre = [&](int c) { return a.s2 + (((size_t)c * a.L2 + (valid ? w2 : 0)) * a.H1 + w1) * a.n3; };
-  copy_fibre_async<LOGN, C::SL>(bufc[0], lt, fibre(0), nload);
+  copy_fibre_async<LOGN, C::N>(bufc[0], lt, fibre(0), nload);
   cp_async_commit();
   load_twiddles<LOGN>(tw, a.tw);
   float2 acc[PER];
@@ -450,7 +350,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3_
   for (int c = 0; c < 3; ++c) {
     float2* buf = bufc[c & 1];
     if (c < 2) {
-      copy_fibre_async<LOGN, C::SL>(bufc[(c + 1) & 1], lt, fibre(c + 1), nload);
+      copy_fibre_async<LOGN, C::N>(bufc[(c + 1) & 1], lt, fibre(c + 1), nload);
       cp_async_commit();
       cp_async_wait<1>();
     } else {
@@ -461,7 +361,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3_
       __syncthreads();
     else
       group_sync<TG>();
-    fwd_fft<LOGN>(buf, lt, tw);
+    fft_pad<LOGN, false>(buf, lt, tw);
     const float* krow = a.kst + (((size_t)c * a.H1 + w1) * a.H2 + (valid ? w2f : 0)) * a.H3;
     const float s2sign = (c == 1 && w2 > a.L2 / 2) ? -1.f : 1.f;
 #pragma unroll
@@ -481,7 +381,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3_
 #pragma unroll
   for (int j = 0; j < PER; ++j) buf[pad16(lt + j * TG)] = acc[j];
   group_sync<TG>();
-  inv_fft<LOGN>(buf, lt, tw);
+  fft_pad<LOGN, true>(buf, lt, tw);
   __syncthreads();  // the transposed store reads every fibre's buffer
   float2* out = a.s1 + (size_t)w1 * a.L2 + (size_t)tile * G;  // S3[i3][w1][w2]
   const int lim = min(G, a.L2 - tile * G);
@@ -492,7 +392,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3_
     const size_t step = (size_t)TG * a.H1 * a.L2;
     float2* dst = out + gg + (size_t)(threadIdx.x / G) * a.H1 * a.L2;
 #pragma unroll 4
-    for (int i3 = threadIdx.x / G; i3 < a.n3; i3 += TG, dst += step) *dst = inv_out<LOGN>(src, i3, tw);
+    for (int i3 = threadIdx.x / G; i3 < a.n3; i3 += TG, dst += step) *dst = src[pad16(i3)];
   }
 }
 
@@ -520,13 +420,13 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3f
   const int nload = valid ? a.n3 : 0;
 #pragma unroll
   for (int c = 0; c < 3; ++c)
-    copy_fibre_async<LOGN, C::SL>(bq[c], lt, a.s2 + (((size_t)c * a.L2 + (valid ? w2 : 0)) * a.H1 + w1) * a.n3, nload);
+    copy_fibre_async<LOGN, C::N>(bq[c], lt, a.s2 + (((size_t)c * a.L2 + (valid ? w2 : 0)) * a.H1 + w1) * a.n3, nload);
   cp_async_commit();
   load_twiddles<LOGN>(tw, a.tw);
   cp_async_wait<0>();
   __syncthreads();
 #pragma unroll
-  for (int c = 0; c < 3; ++c) fwd_fft<LOGN>(bq[c], lt, tw);
+  for (int c = 0; c < 3; ++c) fft_pad<LOGN, false>(bq[c], lt, tw);
   const size_t oct = (size_t)a.H1 * a.H2 * a.H3;
   const float* krow = a.kfield + ((size_t)w1 * a.H2 + (valid ? w2f : 0)) * a.H3;
 #pragma unroll 4
@@ -552,7 +452,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3f
   }
   group_sync<TG>();
 #pragma unroll
-  for (int c = 0; c < 3; ++c) inv_fft<LOGN>(bq[c], lt, tw);
+  for (int c = 0; c < 3; ++c) fft_pad<LOGN, true>(bq[c], lt, tw);
   __syncthreads();  // the transposed stores read every fibre's buffers
   const int lim = min(G, a.L2 - tile * G);
   const int gg = threadIdx.x % G;
@@ -563,7 +463,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK3, LOGN <= 9 ? 2 : 1) fft3d_p3f
       const size_t step = (size_t)TG * a.H1 * a.L2;
       float2* dst = a.s1 + (size_t)c * a.n3 * a.H1 * a.L2 + (size_t)w1 * a.L2 + (size_t)tile * G + gg +
                     (size_t)(threadIdx.x / G) * a.H1 * a.L2;
-      for (int i3 = threadIdx.x / G; i3 < a.n3; i3 += TG, dst += step) *dst = inv_out<LOGN>(src, i3, tw);
+      for (int i3 = threadIdx.x / G; i3 < a.n3; i3 += TG, dst += step) *dst = src[pad16(i3)];
     }
   }
 }
@@ -587,7 +487,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p4_kernel(const __grid_
   const float2* in = a.s1 + (size_t)c * a.n3 * a.H1 * a.L2 + ((size_t)i3 * a.H1 + w1) * a.L2;
   stage_fibre<LOGN, N>(buf, lt, in, w1 < a.H1 ? N : 0);
   __syncthreads();
-  inv_fft<LOGN>(buf, lt, tw);
+  fft_pad<LOGN, true>(buf, lt, tw);
   __syncthreads();  // the transposed store reads every fibre's buffer
   float2* out = a.s2 + (size_t)c * a.n2 * a.n3 * a.H1 + (size_t)i3 * a.H1 + (size_t)tile * G;  // S4[c][i2][i3][w1]
   const int lim = min(G, a.H1 - tile * G);
@@ -597,7 +497,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p4_kernel(const __grid_
     const size_t step = (size_t)TG * a.n3 * a.H1;
     float2* dst = out + gg + (size_t)(threadIdx.x / G) * a.n3 * a.H1;
 #pragma unroll 4
-    for (int i2 = threadIdx.x / G; i2 < a.n2; i2 += TG, dst += step) *dst = inv_out<LOGN>(src, i2, tw);
+    for (int i2 = threadIdx.x / G; i2 < a.n2; i2 += TG, dst += step) *dst = src[pad16(i2)];
   }
 }
 
@@ -647,7 +547,7 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p5_kernel(const __grid_
     }
   }
   __syncthreads();
-  inv_fft<LOGN>(buf, lt, tw);
+  fft_pad<LOGN, true>(buf, lt, tw);
   // fibre f = (c n2 + i2) n3 + i3 -> phi[c][i3][i2][:]
   auto row = [&](int f) {
     const int i3 = f % a.n3, ci2 = f / a.n3;
@@ -657,9 +557,391 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p5_kernel(const __grid_
   float* oa = row(va ? fa : 0);
   float* ob = row(vb ? fa + 1 : 0);
   for (int j = lt; j < a.n1; j += TG) {
-    const float2 v = inv_out<LOGN>(buf, j, tw);
+    const float2 v = buf[pad16(j)];
     if (va) oa[j] = v.x;
     if (vb) ob[j] = v.y;
+  }
+}
+
+// ---------------------------------------------------------------- the passes for lengths 32 to 512
+//
+// A fibre of N = 16 B samples lives in the registers of B lanes (fft.cuh,
+// rf_forward / rf_inverse): it is read from HBM straight into them, crosses
+// shared memory once per transform, and a product with the kernel or the
+// Hermitian extension takes the spectrum in the lanes' frequency order.  With
+// every radix-16 pass (and the staging before it) through shared memory, P3 of
+// 256^3 had its wavefronts 71% and its issue slots 62% busy; it now runs half
+// the wavefronts and waits for HBM.  Before / now, us per pass: 256^3 potential
+// P1 158 / 129, P2 299 / 223 (5.4 TB/s), P3 518 / 448, P4 94 / 82, P5 61 / 47;
+// field P3 of 150 x 100 x 60 (length 128, whose fibres also collided in the
+// banks) 176 / 119.  Registers: 64 at 512 threads (lengths of 512) and 80 at 256
+// keep 32 and 24 warps per SM; P3 takes 128.
+constexpr bool rf_length(int N) { return N >= 32 && N <= 512; }
+template <int LOGN> struct R3 {
+  static constexpr bool OK = rf_length(1 << LOGN);
+  static constexpr int N = 1 << LOGN, B = OK ? N / 16 : 2;
+  static constexpr int G = F3<LOGN>::G, BLOCK = G * B;
+  static constexpr int G3 = F3<LOGN>::G3, BLOCK3 = G3 * B;
+  static constexpr int BS = RegFft<B>::BS;
+  static constexpr size_t smem = (size_t)G * BS * sizeof(float2);
+  static constexpr size_t smem3 = (size_t)(G3 * BS + 24 * BLOCK3) * sizeof(float2);  // and the staged samples
+  static constexpr size_t smem3f = (size_t)3 * G3 * BS * sizeof(float2);
+  static constexpr int MIN = BLOCK >= 512 ? 2 : 3;
+  static constexpr int MIN3 = 2;
+};
+
+// pw[k] = W_N^(l k) from the table [k][l] of exactly rounded values (rf_table_kernel): products of
+// table values (fft.cuh, powers) cost as many instructions as loads and their errors, the same in
+// every fibre, add up coherently (field of 150 x 100 x 60: 5.7e-7 off 64 bits with products, 1.9e-7 with the table)
+template <int B>
+__device__ __forceinline__ void rf_twiddles(const float2* table, int l, float2 (&pw)[16]) {
+#pragma unroll
+  for (int k = 1; k < 16; ++k) pw[k] = __ldg(table + k * B + l);
+}
+
+// table[k][l] = tw[k l], k < 16, l < B = N / 16
+__global__ void rf_table_kernel(int N, const float2* tw, float2* table) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, B = N / 16;
+  if (i < N) table[i] = tw[(i / B) * (i % B)];
+}
+
+// P1 as fft3d_p1_kernel
+template <int LOGN>
+__global__ void __launch_bounds__(R3<LOGN>::BLOCK, R3<LOGN>::MIN) fft3d_p1r_kernel(const __grid_constant__ Fft3dArgs a) {
+  using C = R3<LOGN>;
+  constexpr int N = C::N, B = C::B, G = C::G, BS = C::BS, T = 2 * G;
+  extern __shared__ float2 sm3[];
+  const int g = threadIdx.x / B, l = threadIdx.x % B;
+  float2* buf = sm3 + rf_slot<B>(g) * BS;
+  const int tiles = (a.n2 + T - 1) / T;
+  const int tile = blockIdx.x % tiles;
+  const int ci3 = blockIdx.x / tiles;  // c * n3 + i3
+  const int i2a = tile * T + 2 * g;
+  const float* row = a.m + ((size_t)ci3 * a.n2 + i2a) * a.n1;
+  const bool va = i2a < a.n2, vb = i2a + 1 < a.n2;
+  float2 x[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int j = l + B * r;
+    x[r].x = va && j < a.n1 ? __ldg(row + j) : 0.f;
+    x[r].y = vb && j < a.n1 ? __ldg(row + a.n1 + j) : 0.f;
+  }
+  float2 pw[16], u[16];
+  rf_twiddles<B>(a.tw, l, pw);
+  rf_forward<B>(x, u, buf, l, pw);
+#pragma unroll
+  for (int s = 0; s < 16; ++s) buf[rf_freq<B>(l, s)] = u[s];
+  __syncthreads();  // the split step reads every fibre pair's buffer
+  const int c = ci3 / a.n3, i3 = ci3 % a.n3;
+  float2* out = a.s1 + (size_t)c * a.H1 * a.n3 * a.n2 + (size_t)i3 * a.n2 + (size_t)tile * T;
+  const int lim = min(T, a.n2 - tile * T);
+  // X_a = (Z_w + conj Z_{N-w}) / 2, X_b = (Z_w - conj Z_{N-w}) / 2i; stored at S1[c][w][i3][i2]
+  constexpr int WS = C::BLOCK / T > 0 ? C::BLOCK / T : 1;
+  for (int g2 = threadIdx.x % T; g2 < T; g2 += C::BLOCK) {
+    if (g2 >= lim) continue;
+    const float2* b = sm3 + rf_slot<B>(g2 >> 1) * BS;
+    const size_t step = (size_t)WS * a.n3 * a.n2;
+    const int w0 = C::BLOCK >= T ? threadIdx.x / T : 0;
+    float2* dst = out + g2 + (size_t)w0 * a.n3 * a.n2;
+#pragma unroll 4
+    for (int w = w0; w < a.H1; w += WS, dst += step) {
+      const float2 Z = b[w], Zc = b[(N - w) & (N - 1)];
+      *dst = (g2 & 1) ? make_float2(0.5f * (Z.y + Zc.y), -0.5f * (Z.x - Zc.x))
+                      : make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y - Zc.y));
+    }
+  }
+}
+
+// P2 as fft3d_p2_kernel
+template <int LOGN>
+__global__ void __launch_bounds__(R3<LOGN>::BLOCK, R3<LOGN>::MIN) fft3d_p2r_kernel(const __grid_constant__ Fft3dArgs a) {
+  using C = R3<LOGN>;
+  constexpr int N = C::N, B = C::B, G = C::G, BS = C::BS;
+  extern __shared__ float2 sm3[];
+  const int g = threadIdx.x / B, l = threadIdx.x % B;
+  float2* buf = sm3 + rf_slot<B>(g) * BS;
+  const int tiles = (a.n3 + G - 1) / G;
+  const int tile = blockIdx.x % tiles;
+  const int cw1 = blockIdx.x / tiles;  // c * H1 + w1
+  const int i3 = tile * G + g;
+  const float2* in = a.s1 + ((size_t)cw1 * a.n3 + i3) * a.n2;
+  const int n = i3 < a.n3 ? a.n2 : 0;
+  float2 x[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) x[r] = l + B * r < n ? __ldg(in + l + B * r) : make_float2(0.f, 0.f);
+  float2 pw[16], u[16];
+  rf_twiddles<B>(a.tw, l, pw);
+  rf_forward<B>(x, u, buf, l, pw);
+#pragma unroll
+  for (int s = 0; s < 16; ++s) buf[rf_freq<B>(l, s)] = u[s];
+  __syncthreads();  // the transposed store reads every fibre's buffer
+  const int c = cw1 / a.H1, w1 = cw1 % a.H1;
+  float2* out = a.s2 + (size_t)c * a.L2 * a.H1 * a.n3 + (size_t)w1 * a.n3 + (size_t)tile * G;
+  const int lim = min(G, a.n3 - tile * G);
+  const int gg = threadIdx.x % G;
+  if (gg < lim) {
+    const float2* src = sm3 + rf_slot<B>(gg) * BS;
+    const size_t step = (size_t)B * a.H1 * a.n3;
+    float2* dst = out + gg + (size_t)(threadIdx.x / G) * a.H1 * a.n3;
+#pragma unroll 4
+    for (int w2 = threadIdx.x / G; w2 < N; w2 += B, dst += step) *dst = src[w2];
+  }
+}
+
+// P3 as fft3d_p3_kernel.  All three components' fibres are copied to shared
+// memory at once (cp.async, each lane its own samples), and a component's
+// kernel entries are read into registers before its transform: with 16 warps
+// per SM (128 registers) loads left where they are used cost as much time as
+// the transforms.
+template <int LOGN>
+__global__ void __launch_bounds__(R3<LOGN>::BLOCK3, 2) fft3d_p3r_kernel(const __grid_constant__ Fft3dArgs a) {
+  using C = R3<LOGN>;
+  constexpr int N = C::N, B = C::B, G = C::G3, BS = C::BS;
+  extern __shared__ float2 sm3[];
+  const int g = threadIdx.x / B, l = threadIdx.x % B;
+  float2* buf = sm3 + rf_slot<B>(g) * BS;
+  float2* stage = sm3 + G * BS + threadIdx.x;  // sample (c, r) of this lane at (8 c + r) BLOCK3
+  const int tiles = (a.L2 + G - 1) / G;
+  const int tile = blockIdx.x % tiles;
+  const int w1 = blockIdx.x / tiles;
+  const int w2 = tile * G + g;
+  const bool valid = w2 < a.L2;
+  const int w2f = w2 <= a.L2 / 2 ? w2 : a.L2 - w2;
+  const int n = valid ? a.n3 : 0;
+  {
+    const float2* in = a.s2 + ((size_t)(valid ? w2 : 0) * a.H1 + w1) * a.n3;
+    const size_t cstep = (size_t)a.L2 * a.H1 * a.n3;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const bool ok = l + B * r < n;
+        cp_async8(stage + (8 * c + r) * C::BLOCK3, ok ? in + c * cstep + l + B * r : in, ok);
+      }
+      cp_async_commit();
+    }
+  }
+  float2 acc[16], pw[16];
+  rf_twiddles<B>(a.tw, l, pw);
+  const float* krow = a.kst + ((size_t)w1 * a.H2 + (valid ? w2f : 0)) * a.H3;
+  const size_t kstep = (size_t)a.H1 * a.H2 * a.H3;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float kv[16];
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+      const int w3 = rf_freq<B>(l, s);
+      kv[s] = __ldg(krow + c * kstep + (w3 > N / 2 ? N - w3 : w3));
+    }
+    if (c == 0) cp_async_wait<2>();
+    if (c == 1) cp_async_wait<1>();
+    if (c == 2) cp_async_wait<0>();
+    float2 x[8], u[16];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) x[r] = stage[(8 * c + r) * C::BLOCK3];  // this lane's own copies
+    rf_forward<B>(x, u, buf, l, pw);
+    const bool flip2 = c == 1 && w2 > a.L2 / 2;
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+      float kvs = kv[s];
+      if (c == 2 ? rf_freq<B>(l, s) > N / 2 : flip2) kvs = -kvs;
+      // (i kv) Z
+      if (c == 0) {
+        acc[s] = make_float2(-kvs * u[s].y, kvs * u[s].x);
+      } else {
+        acc[s].x = fmaf(-kvs, u[s].y, acc[s].x);
+        acc[s].y = fmaf(kvs, u[s].x, acc[s].y);
+      }
+    }
+  }
+  float2 v[16];
+  rf_inverse<B>(acc, v, buf, l, pw);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) buf[l + B * r] = v[r];
+  __syncthreads();  // the transposed store reads every fibre's buffer
+  float2* out = a.s1 + (size_t)w1 * a.L2 + (size_t)tile * G;  // S3[i3][w1][w2]
+  const int lim = min(G, a.L2 - tile * G);
+  const int gg = threadIdx.x % G;
+  if (gg < lim) {
+    const float2* src = sm3 + rf_slot<B>(gg) * BS;
+    const size_t step = (size_t)B * a.H1 * a.L2;
+    float2* dst = out + gg + (size_t)(threadIdx.x / G) * a.H1 * a.L2;
+#pragma unroll 4
+    for (int i3 = threadIdx.x / G; i3 < a.n3; i3 += B, dst += step) *dst = src[i3];
+  }
+}
+
+// P3 of the stray field as fft3d_p3f_kernel: the spectra of components 0 and 1
+// wait in shared memory (each lane's own slots) while component 2's is formed,
+// and each bin's three outputs replace its inputs
+template <int LOGN>
+__global__ void __launch_bounds__(R3<LOGN>::BLOCK3, R3<LOGN>::MIN3) fft3d_p3fr_kernel(const __grid_constant__ Fft3dArgs a) {
+  using C = R3<LOGN>;
+  constexpr int N = C::N, B = C::B, G = C::G3, BS = C::BS;
+  extern __shared__ float2 sm3[];
+  const int g = threadIdx.x / B, l = threadIdx.x % B;
+  float2* bq[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) bq[c] = sm3 + (c * G + rf_slot<B>(g)) * BS;
+  const int tiles = (a.L2 + G - 1) / G;
+  const int tile = blockIdx.x % tiles;
+  const int w1 = blockIdx.x / tiles;
+  const int w2 = tile * G + g;
+  const bool valid = w2 < a.L2;
+  const bool m2 = w2 > a.L2 / 2;
+  const int w2f = m2 ? a.L2 - w2 : w2;
+  const int n = valid ? a.n3 : 0;
+  const float2* in = a.s2 + ((size_t)(valid ? w2 : 0) * a.H1 + w1) * a.n3;
+  const size_t cstep = (size_t)a.L2 * a.H1 * a.n3;
+  float2 x[8], u[16], pw[16];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) x[r] = l + B * r < n ? __ldg(in + l + B * r) : make_float2(0.f, 0.f);
+  rf_twiddles<B>(a.tw, l, pw);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float2 nx[8];
+    if (c < 2) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        nx[r] = l + B * r < n ? __ldg(in + (c + 1) * cstep + l + B * r) : make_float2(0.f, 0.f);
+    }
+    rf_forward<B>(x, u, bq[c], l, pw);
+    if (c < 2) {
+#pragma unroll
+      for (int s = 0; s < 16; ++s) bq[c][rf_freq<B>(l, s)] = u[s];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) x[r] = nx[r];
+    }
+  }
+  const size_t oct = (size_t)a.H1 * a.H2 * a.H3;
+  const float* krow = a.kfield + ((size_t)w1 * a.H2 + (valid ? w2f : 0)) * a.H3;
+#pragma unroll
+  for (int s = 0; s < 16; ++s) {
+    const int w3 = rf_freq<B>(l, s);
+    const bool m3 = w3 > N / 2;
+    const int w3f = m3 ? N - w3 : w3;
+    const float k00 = __ldg(krow + w3f), k11 = __ldg(krow + oct + w3f), k22 = __ldg(krow + 2 * oct + w3f);
+    float k01 = __ldg(krow + 3 * oct + w3f), k02 = __ldg(krow + 4 * oct + w3f), k12 = __ldg(krow + 5 * oct + w3f);
+    if (m2) {
+      k01 = -k01;
+      k12 = -k12;
+    }
+    if (m3) {
+      k02 = -k02;
+      k12 = -k12;
+    }
+    const float2 x0 = bq[0][w3], x1 = bq[1][w3], x2 = u[s];
+    bq[0][w3] = make_float2(k00 * x0.x + k01 * x1.x + k02 * x2.x, k00 * x0.y + k01 * x1.y + k02 * x2.y);
+    bq[1][w3] = make_float2(k01 * x0.x + k11 * x1.x + k12 * x2.x, k01 * x0.y + k11 * x1.y + k12 * x2.y);
+    u[s] = make_float2(k02 * x0.x + k12 * x1.x + k22 * x2.x, k02 * x0.y + k12 * x1.y + k22 * x2.y);
+  }
+#pragma unroll
+  for (int c = 2; c >= 0; --c) {
+    if (c < 2) {
+#pragma unroll
+      for (int s = 0; s < 16; ++s) u[s] = bq[c][rf_freq<B>(l, s)];
+      __syncwarp();  // the exchange overwrites other lanes' bins
+    }
+    float2 v[16];
+    rf_inverse<B>(u, v, bq[c], l, pw);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) bq[c][l + B * r] = v[r];
+  }
+  __syncthreads();  // the transposed stores read every fibre's buffers
+  const int lim = min(G, a.L2 - tile * G);
+  const int gg = threadIdx.x % G;
+  if (gg < lim) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float2* src = sm3 + (c * G + rf_slot<B>(gg)) * BS;
+      const size_t step = (size_t)B * a.H1 * a.L2;
+      float2* dst = a.s1 + (size_t)c * a.n3 * a.H1 * a.L2 + (size_t)w1 * a.L2 + (size_t)tile * G + gg +
+                    (size_t)(threadIdx.x / G) * a.H1 * a.L2;
+#pragma unroll 4
+      for (int i3 = threadIdx.x / G; i3 < a.n3; i3 += B, dst += step) *dst = src[i3];
+    }
+  }
+}
+
+// P4 as fft3d_p4_kernel
+template <int LOGN>
+__global__ void __launch_bounds__(R3<LOGN>::BLOCK, R3<LOGN>::MIN) fft3d_p4r_kernel(const __grid_constant__ Fft3dArgs a) {
+  using C = R3<LOGN>;
+  constexpr int B = C::B, G = C::G, BS = C::BS;
+  extern __shared__ float2 sm3[];
+  const int g = threadIdx.x / B, l = threadIdx.x % B;
+  float2* buf = sm3 + rf_slot<B>(g) * BS;
+  const int tiles = (a.H1 + G - 1) / G;
+  const int tile = blockIdx.x % tiles;
+  const int ci3 = blockIdx.x / tiles;  // c * n3 + i3
+  const int c = ci3 / a.n3, i3 = ci3 % a.n3;
+  const int w1 = tile * G + g;
+  const float2* in = a.s1 + (size_t)c * a.n3 * a.H1 * a.L2 + ((size_t)i3 * a.H1 + w1) * a.L2;
+  float2 u[16], v[16], pw[16];
+#pragma unroll
+  for (int s = 0; s < 16; ++s) u[s] = w1 < a.H1 ? __ldg(in + rf_freq<B>(l, s)) : make_float2(0.f, 0.f);
+  rf_twiddles<B>(a.tw, l, pw);
+  rf_inverse<B>(u, v, buf, l, pw);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) buf[l + B * r] = v[r];
+  __syncthreads();  // the transposed store reads every fibre's buffer
+  float2* out = a.s2 + (size_t)c * a.n2 * a.n3 * a.H1 + (size_t)i3 * a.H1 + (size_t)tile * G;  // S4[c][i2][i3][w1]
+  const int lim = min(G, a.H1 - tile * G);
+  const int gg = threadIdx.x % G;
+  if (gg < lim) {
+    const float2* src = sm3 + rf_slot<B>(gg) * BS;
+    const size_t step = (size_t)B * a.n3 * a.H1;
+    float2* dst = out + gg + (size_t)(threadIdx.x / G) * a.n3 * a.H1;
+#pragma unroll 4
+    for (int i2 = threadIdx.x / G; i2 < a.n2; i2 += B, dst += step) *dst = src[i2];
+  }
+}
+
+// P5 as fft3d_p5_kernel
+template <int LOGN>
+__global__ void __launch_bounds__(R3<LOGN>::BLOCK, R3<LOGN>::MIN) fft3d_p5r_kernel(const __grid_constant__ Fft3dArgs a) {
+  using C = R3<LOGN>;
+  constexpr int N = C::N, B = C::B, G = C::G, BS = C::BS, T = 2 * G;
+  extern __shared__ float2 sm3[];
+  const int g = threadIdx.x / B, l = threadIdx.x % B;
+  float2* buf = sm3 + rf_slot<B>(g) * BS;
+  const int nf = a.nco * a.n2 * a.n3;
+  const int fa = blockIdx.x * T + 2 * g;
+  const bool va = fa < nf, vb = fa + 1 < nf;
+  const float2* ina = a.s2 + (size_t)fa * a.H1;
+  const float2* inb = ina + a.H1;
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 u[16], v[16], pw[16];
+#pragma unroll
+  for (int s = 0; s < 16; ++s) {
+    const int w = rf_freq<B>(l, s);
+    const int src = w <= N / 2 ? w : N - w;
+    float2 xa = va ? __ldg(ina + src) : zero, xb = vb ? __ldg(inb + src) : zero;
+    // Hermitian extension X_w = conj X_{N-w}; the imaginary parts at w = 0, N/2 are dropped
+    if (w > N / 2) {
+      xa.y = -xa.y;
+      xb.y = -xb.y;
+    }
+    if (w == 0 || w == N / 2) xa.y = xb.y = 0.f;
+    u[s] = make_float2(xa.x - xb.y, xa.y + xb.x);  // X_a + i X_b
+  }
+  rf_twiddles<B>(a.tw, l, pw);
+  rf_inverse<B>(u, v, buf, l, pw);
+  // fibre f = (c n2 + i2) n3 + i3 -> phi[c][i3][i2][:]
+  auto row = [&](int f) {
+    const int i3 = f % a.n3, ci2 = f / a.n3;
+    const int i2 = ci2 % a.n2, c = ci2 / a.n2;
+    return a.phi + (((size_t)c * a.n3 + i3) * a.n2 + i2) * a.n1;
+  };
+  float* oa = row(va ? fa : 0);
+  float* ob = row(vb ? fa + 1 : 0);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int j = l + B * r;
+    if (j < a.n1) {
+      if (va) oa[j] = v[r].x;
+      if (vb) ob[j] = v[r].y;
+    }
   }
 }
 
@@ -758,6 +1040,8 @@ struct Fft3dState {
   float* kst = nullptr;
   float* kfield = nullptr;  // stray-field kernels, built on first use
   float* hfield = nullptr;  // [3][n3][n2][n1] field scratch of the energy
+  float2* table = nullptr;  // twiddle tables [16][L_p / 16] of the axes whose passes run in registers
+  const float2* tw[3];      // each axis' twiddles as its passes read them
   float2* s1 = nullptr;
   float2* s2 = nullptr;
   size_t s1_elems = 0, s2_elems = 0;
@@ -772,32 +1056,41 @@ static int log2_exact(int v) {
 template <int LOGN>
 static demag_status launch_pass(demag_plan* P, int pass, const Fft3dArgs& a, int blocks, cudaStream_t st) {
   using C = F3<LOGN>;
-  // pass 6 is the P3 of the stray field
-  const void* fn = pass == 1 ? (const void*)fft3d_p1_kernel<LOGN>
-                 : pass == 2 ? (const void*)fft3d_p2_kernel<LOGN>
-                 : pass == 3 ? (const void*)fft3d_p3_kernel<LOGN>
-                 : pass == 4 ? (const void*)fft3d_p4_kernel<LOGN>
-                 : pass == 5 ? (const void*)fft3d_p5_kernel<LOGN>
-                             : (const void*)fft3d_p3f_kernel<LOGN>;
+  using R = R3<LOGN>;
+  // lengths 32 to 512 in registers, the others by in-place passes; pass 6 is the P3 of the stray field
+  using Fn = void (*)(const Fft3dArgs);
+  const int i = pass - 1;
+  Fn fn[6];
+  int block[6];
+  size_t smem[6];
+  if constexpr (R::OK) {
+    const Fn f[6] = {fft3d_p1r_kernel<LOGN>, fft3d_p2r_kernel<LOGN>, fft3d_p3r_kernel<LOGN>,
+                     fft3d_p4r_kernel<LOGN>, fft3d_p5r_kernel<LOGN>, fft3d_p3fr_kernel<LOGN>};
+    for (int k = 0; k < 6; ++k) {
+      fn[k] = f[k];
+      block[k] = k == 2 || k == 5 ? R::BLOCK3 : R::BLOCK;
+      smem[k] = k == 2 ? R::smem3 : k == 5 ? R::smem3f : R::smem;
+    }
+  } else {
+    const Fn f[6] = {fft3d_p1_kernel<LOGN>, fft3d_p2_kernel<LOGN>, fft3d_p3_kernel<LOGN>,
+                     fft3d_p4_kernel<LOGN>, fft3d_p5_kernel<LOGN>, fft3d_p3f_kernel<LOGN>};
+    for (int k = 0; k < 6; ++k) {
+      fn[k] = f[k];
+      block[k] = k == 2 || k == 5 ? C::BLOCK3 : C::BLOCK;
+      smem[k] = k == 2 ? C::smem3 : k == 5 ? C::smem3f : C::smem;
+    }
+  }
   // the attribute is set on first use per kernel and device (so that later
   // launches, e.g. under stream capture, make no attribute calls)
-  static unsigned long long done[7] = {0, 0, 0, 0, 0, 0, 0};
+  static unsigned long long done[6] = {0, 0, 0, 0, 0, 0};
   int dev = 0;
   cudaGetDevice(&dev);
   const unsigned long long bit = 1ull << (dev & 63);
-  const size_t smem = pass == 3 ? C::smem3 : (pass == 6 ? C::smem3f : C::smem);
-  if (smem > 48 * 1024 && !(done[pass] & bit)) {
-    DEMAG_CUDA(P, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    done[pass] |= bit;
+  if (smem[i] > 48 * 1024 && !(done[i] & bit)) {
+    DEMAG_CUDA(P, cudaFuncSetAttribute((const void*)fn[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem[i]));
+    done[i] |= bit;
   }
-  switch (pass) {
-    case 1: DEMAG_LAUNCH(P, kFamFFT3D, st, fft3d_p1_kernel<LOGN><<<blocks, C::BLOCK, C::smem, st>>>(a)); break;
-    case 2: DEMAG_LAUNCH(P, kFamFFT3D, st, fft3d_p2_kernel<LOGN><<<blocks, C::BLOCK, C::smem, st>>>(a)); break;
-    case 3: DEMAG_LAUNCH(P, kFamFFT3D, st, fft3d_p3_kernel<LOGN><<<blocks, C::BLOCK3, C::smem3, st>>>(a)); break;
-    case 4: DEMAG_LAUNCH(P, kFamFFT3D, st, fft3d_p4_kernel<LOGN><<<blocks, C::BLOCK, C::smem, st>>>(a)); break;
-    case 5: DEMAG_LAUNCH(P, kFamFFT3D, st, fft3d_p5_kernel<LOGN><<<blocks, C::BLOCK, C::smem, st>>>(a)); break;
-    default: DEMAG_LAUNCH(P, kFamFFT3D, st, fft3d_p3f_kernel<LOGN><<<blocks, C::BLOCK3, C::smem3f, st>>>(a)); break;
-  }
+  DEMAG_LAUNCH(P, kFamFFT3D, st, fn[i]<<<blocks, block[i], smem[i], st>>>(a));
   DEMAG_LAUNCHED(P, "fft3d pass");
   return DEMAG_OK;
 }
@@ -846,6 +1139,7 @@ demag_status fft3d_prepare(demag_plan* P, cudaStream_t st) {
     cudaFree(S->kst);
     cudaFree(S->s1);
     cudaFree(S->s2);
+    cudaFree(S->table);
     delete S;
     return cuda_error(P, e, what);
   };
@@ -866,6 +1160,16 @@ demag_status fft3d_prepare(demag_plan* P, cudaStream_t st) {
                  fft3d_kernel_kernel<<<3 * H1 * H2, 256, 0, st>>>(P->M, hstride, H1, H2, H3, P->scale, sym,
                                                                   S->kst));
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "fft3d_kernel_kernel");
+  }
+  if ((e = cudaMalloc(&S->table, sizeof(float2) * ((size_t)L1 + L2 + L3))) != cudaSuccess)
+    return fail(e, "malloc twiddle tables");
+  for (int p = 0, at = 0; p < 3; at += P->L[p], ++p) {
+    S->tw[p] = P->twid[p];
+    if (!rf_length(P->L[p])) continue;
+    S->tw[p] = S->table + at;
+    DEMAG_LAUNCH(P, kFamSetup, st,
+                 rf_table_kernel<<<(P->L[p] + 255) / 256, 256, 0, st>>>(P->L[p], P->twid[p], S->table + at));
+    if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "rf_table_kernel");
   }
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return fail(e, "fft3d setup");
   cudaFree(sym);
@@ -932,6 +1236,7 @@ void fft3d_destroy(demag_plan* P) {
   cudaFree(S->kst);
   cudaFree(S->s1);
   cudaFree(S->s2);
+  cudaFree(S->table);
   delete S;
   P->f3 = nullptr;
 }
@@ -962,15 +1267,15 @@ static demag_status fft3d_run(demag_plan* P, const float* m, float* out, bool fi
   const int l1 = S->logL[0], l2 = S->logL[1], l3 = S->logL[2];
   const int G1 = f3_fibres(1 << l1), G2 = f3_fibres(1 << l2), G3 = f3_fibres_p3(1 << l3);
   auto cdiv = [](long x, long y) { return (int)((x + y - 1) / y); };
-  a.tw = P->twid[0];
+  a.tw = S->tw[0];
   if ((rc = dispatch_pass(P, l1, 1, a, 3 * a.n3 * cdiv(a.n2, 2 * G1), st)) != DEMAG_OK) return rc;
-  a.tw = P->twid[1];
+  a.tw = S->tw[1];
   if ((rc = dispatch_pass(P, l2, 2, a, 3 * a.H1 * cdiv(a.n3, G2), st)) != DEMAG_OK) return rc;
-  a.tw = P->twid[2];
+  a.tw = S->tw[2];
   if ((rc = dispatch_pass(P, l3, field ? 6 : 3, a, a.H1 * cdiv(a.L2, G3), st)) != DEMAG_OK) return rc;
-  a.tw = P->twid[1];
+  a.tw = S->tw[1];
   if ((rc = dispatch_pass(P, l2, 4, a, a.nco * a.n3 * cdiv(a.H1, G2), st)) != DEMAG_OK) return rc;
-  a.tw = P->twid[0];
+  a.tw = S->tw[0];
   return dispatch_pass(P, l1, 5, a, cdiv((long)a.nco * a.n2 * a.n3, 2 * G1), st);
 }
 

@@ -98,35 +98,6 @@ struct TwN {
   __device__ __forceinline__ float2 operator()(int m) const { return s.L(2 * m); }
 };
 
-// The first 8 outputs of an inverse 16-point DFT (the kept half of the last
-// pass): two 8-point DFTs of the even and odd inputs and the "+" half of the
-// final butterflies.
-template <int K>
-__device__ __forceinline__ void combine_half16(float2 (&v)[16], float2 (&e)[8], float2 (&o)[8]) {
-  if constexpr (K < 8) {
-    const float2 t = rot<16, K, true>(o[K]);
-    if constexpr (K == 4) {  // +i: folded into scalar adds
-      v[K].x = e[K].x + t.x;
-      v[K].y = e[K].y + t.y;
-    } else {
-      v[K] = cadd(e[K], t);
-    }
-    combine_half16<K + 1>(v, e, o);
-  }
-}
-
-__device__ __forceinline__ void idft16_first_half(float2 (&v)[16]) {
-  float2 e[8], o[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    e[i] = v[2 * i];
-    o[i] = v[2 * i + 1];
-  }
-  dft_reg<8, true>(e);
-  dft_reg<8, true>(o);
-  combine_half16<0>(v, e, o);
-}
-
 // In-place middle pass of radix R on the padded buffer (inverse direction):
 // every item is read into registers, the block synchronises, then writes.
 template <int R, int N, int TG>
