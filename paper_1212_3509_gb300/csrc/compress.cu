@@ -41,6 +41,7 @@ struct Compressed {
   double* cgen = nullptr;   // [rhomax][3 q][3 p][glen] compressed generators
   float* csym = nullptr;    // [rhomax][3][3][Lmax/2 + 1]
   float2* cpair = nullptr;  // [rhomax][3][3][Lmax/2]
+  float* creg = nullptr;    // [rhomax][3][3][Lmax] in thread order (symreg_at), behind cpair
   float* core = nullptr;    // [3 q][rho3][rho2][rho1]
 };
 
@@ -769,6 +770,7 @@ bool compressed_view(const demag_plan* P, CompressedView* v) {
   if (!C) return false;
   for (int p = 0; p < 3; ++p) v->rho[p] = C->rho[p];
   v->cpair = C->cpair;
+  v->creg = C->creg;
   v->core = C->core;
   return true;
 }
@@ -887,7 +889,10 @@ extern "C" demag_status demag_compress_kernel(demag_plan* P, double tol, void* s
   const int symstride = P->Lmax / 2 + 1, pairstride = P->Lmax / 2;
   CMP_CUDA(cudaMalloc(&C->csym, sizeof(float) * (size_t)rmax * 9 * symstride));
   CMP_CUDA(cudaMemsetAsync(C->csym, 0, sizeof(float) * (size_t)rmax * 9 * symstride, st));
-  CMP_CUDA(cudaMalloc(&C->cpair, sizeof(float2) * (size_t)rmax * 9 * pairstride));
+  const size_t pairs = (size_t)rmax * 9 * pairstride;
+  const bool regs = any_toep_in_registers(P);
+  CMP_CUDA(cudaMalloc(&C->cpair, sizeof(float2) * (regs ? 2 : 1) * pairs));
+  if (regs) C->creg = reinterpret_cast<float*>(C->cpair + pairs);
   for (int p = 0; p < 3; ++p) {
     dispatch_symbol(P, p, C->rho[p], 3, C->cgen, C->csym, st);
     CMP_CUDA(cudaGetLastError());
@@ -897,7 +902,7 @@ extern "C" demag_status demag_compress_kernel(demag_plan* P, double tol, void* s
     if (blocks > 152 * 16) blocks = 152 * 16;
     DEMAG_LAUNCH(P, kFamSetup, st,
                  sympair_kernel<<<(int)blocks, 256, 0, st>>>(C->rho[p], 3, p, N, symstride, pairstride, C->csym,
-                                                             C->cpair));
+                                                             C->cpair, C->creg));
     CMP_CUDA(cudaGetLastError());
   }
   CMP_CUDA(cudaStreamSynchronize(st));

@@ -273,17 +273,9 @@ __device__ __forceinline__ void rf_part(float2 (&u)[16], float2 (&send)[8], floa
   }
 }
 
-// x: the 8 time samples x[l + B r]; u: the spectrum in frequency order.  pw[r] = W_N^(l r).
+// Forward: the twiddled 16-point DFTs lie in buf (row k1, column l); u: the spectrum in frequency order.
 template <int B>
-__device__ __forceinline__ void rf_forward(const float2 (&x)[8], float2 (&u)[16], float2* buf, int l,
-                                           const float2 (&pw)[16]) {
-  {
-    float2 v[16];
-    dft16_of_half(x, v);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) buf[k * (B + 1) + l] = k ? cmul(v[k], pw[k]) : v[k];
-  }
-  __syncwarp();
+__device__ __forceinline__ void rf_finish(float2 (&u)[16], float2* buf, int l) {
   if constexpr (B == 32) {
     const int k1 = l & 15, h = l >> 4;
 #pragma unroll
@@ -309,10 +301,23 @@ __device__ __forceinline__ void rf_forward(const float2 (&x)[8], float2 (&u)[16]
   }
 }
 
-// u: a spectrum in frequency order; v[r], r < 8: x[l + B r] of the unnormalised inverse.
+// x: the 8 time samples x[l + B r]; u: the spectrum in frequency order.  pw[r] = W_N^(l r).
 template <int B>
-__device__ __forceinline__ void rf_inverse(float2 (&u)[16], float2 (&v)[16], float2* buf, int l,
+__device__ __forceinline__ void rf_forward(const float2 (&x)[8], float2 (&u)[16], float2* buf, int l,
                                            const float2 (&pw)[16]) {
+  {
+    float2 v[16];
+    dft16_of_half(x, v);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) buf[k * (B + 1) + l] = k ? cmul(v[k], pw[k]) : v[k];
+  }
+  __syncwarp();
+  rf_finish<B>(u, buf, l);
+}
+
+// u: a spectrum in frequency order; its inverse B-point DFTs are left in buf (row k1, column l).
+template <int B>
+__device__ __forceinline__ void rf_begin(float2 (&u)[16], float2* buf, int l) {
   if constexpr (B == 32) {
     const int k1 = l & 15, h = l >> 4;
     float2 send[8], keep[8];
@@ -338,6 +343,13 @@ __device__ __forceinline__ void rf_inverse(float2 (&u)[16], float2 (&v)[16], flo
       for (int j = 0; j < B; ++j) buf[(l + B * e) * (B + 1) + j] = w[j];
     }
   }
+}
+
+// u: a spectrum in frequency order; v[r], r < 8: x[l + B r] of the unnormalised inverse.
+template <int B>
+__device__ __forceinline__ void rf_inverse(float2 (&u)[16], float2 (&v)[16], float2* buf, int l,
+                                           const float2 (&pw)[16]) {
+  rf_begin<B>(u, buf, l);
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
@@ -346,6 +358,56 @@ __device__ __forceinline__ void rf_inverse(float2 (&u)[16], float2 (&v)[16], flo
   }
   __syncwarp();
   idft16_first_half(v);
+}
+
+// Inverse 16-point DFT of w^k v[k] with the powers of w inside its radix-2 steps: eight twiddles
+// (16 registers) where separate products keep fifteen.  Outputs r < 8 only with HALF.
+struct Twid16 {
+  float2 a[4];  // w exp(2 pi i j / 16)
+  float2 b[2];  // w^2 exp(2 pi i j / 8)
+  float2 c, d;  // w^4, w^8
+};
+
+template <int R, int K>
+__device__ __forceinline__ float2 tw16_rot(const Twid16& t, float2 v) {
+  constexpr int j = K % (R >= 4 ? R / 4 : 1);
+  if constexpr (R == 16) return cmul(v, t.a[j]);
+  if constexpr (R == 8) return cmul(v, t.b[j]);
+  if constexpr (R == 4) return cmul(v, t.c);
+  return cmul(v, t.d);
+}
+template <int R, int K, bool HALF>
+__device__ __forceinline__ void tw16_combine(const Twid16& t, const float2 (&e)[R / 2], const float2 (&o)[R / 2],
+                                             float2 (&v)[R]) {
+  if constexpr (K < R / 2) {
+    const float2 p = tw16_rot<R, K>(t, o[K]);
+    if constexpr (R >= 4 && K >= R / 4) {  // a further factor i
+      v[K].x = e[K].x - p.y;
+      v[K].y = e[K].y + p.x;
+      if constexpr (!HALF) {
+        v[K + R / 2].x = e[K].x + p.y;
+        v[K + R / 2].y = e[K].y - p.x;
+      }
+    } else {
+      v[K] = cadd(e[K], p);
+      if constexpr (!HALF) v[K + R / 2] = csub(e[K], p);
+    }
+    tw16_combine<R, K + 1, HALF>(t, e, o, v);
+  }
+}
+template <int R, bool HALF>
+__device__ __forceinline__ void tw16_idft(const Twid16& t, float2 (&v)[R]) {
+  if constexpr (R > 1) {
+    float2 e[R / 2], o[R / 2];
+#pragma unroll
+    for (int i = 0; i < R / 2; ++i) {
+      e[i] = v[2 * i];
+      o[i] = v[2 * i + 1];
+    }
+    tw16_idft<R / 2, false>(t, e);
+    tw16_idft<R / 2, false>(t, o);
+    tw16_combine<R, 0, HALF>(t, e, o, v);
+  }
 }
 
 // Radix plan for N = 2^LOGN: number of radix-16 passes and the remainder radix.

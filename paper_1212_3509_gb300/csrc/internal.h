@@ -49,6 +49,7 @@ struct demag_plan {
   float* sym = nullptr;      // [M][2][3][Lmax/2 + 1] symbols / L_p
   float2* twid[3] = {nullptr, nullptr, nullptr};  // per axis: exp(-2 pi i m / L_p), m < L_p
   float2* sympair = nullptr; // [M][2][3][Lmax/2]: (symbol[f], symbol[L_p/2 - f]) for f < L_p/2
+  float* symreg = nullptr;   // [M][2][3][Lmax]: all L_p symbol values in thread order (symreg_at), behind sympair
   double* scale = nullptr;   // [M]: c * s * omega_k
   double* gend = nullptr;    // [M][2][3][glen]: derivative generators dE/s, dF/s (lazily, analytic stray field)
 
@@ -187,6 +188,7 @@ void tc_destroy(demag_plan* plan);
 struct CompressedView {
   int rho[3];
   const float2* cpair;  // symbol pairs [rhomax][3 q][3 p][Lmax/2]
+  const float* creg;    // all symbol values in thread order [rhomax][3 q][3 p][Lmax]
   const float* core;    // [3 q][rho3][rho2][rho1]
 };
 bool compressed_view(const demag_plan* plan, CompressedView* v);
@@ -207,8 +209,23 @@ __global__ void nodes_kernel(int M, double c0, double cscale, double* nodes, dou
 __global__ void generators_kernel(int M, int glen, GridInfo g, const double* nodes, double* gen);
 demag_status require_uniform(demag_plan* plan, const char* what);
 void dispatch_symbol(demag_plan* P, int axis, int M, int nsets, const double* gen, float* sym, cudaStream_t st);
+// Axes whose circulant transform the structured kernel keeps in registers: L = 2N of 512 to 4096 points.
+// Against in-place passes (CP, r = 4, 64 items, GB300): n = 200 38 against 70 us, 1024 150 against 241,
+// 2048 355 against 418; at n = 4096 a column takes 512 threads, one block per SM, whose barriers nothing
+// covers: 873 against 796 us (922 with two threads per last step), so it ends at 2048.
+__host__ __device__ inline bool toep_in_registers(int N) { return N >= 256 && N <= 2048; }
+inline bool any_toep_in_registers(const demag_plan* P) {
+  return toep_in_registers(P->L[0] / 2) || toep_in_registers(P->L[1] / 2) || toep_in_registers(P->L[2] / 2);
+}
+// Place of symbol value f < L in the order of that kernel's threads: thread f1 B + l (B = L / 256,
+// f = f1 + 16 f2) holds element s of its group's spectrum (rf_freq), four elements to a 16-byte load.
+__host__ __device__ inline int symreg_at(int f, int L) {
+  const int B = L / 256, f1 = f & 15, lo = (f >> 4) & 15, c = f >> 8;
+  const int l = lo % B, s = (lo / B) * B + c;
+  return ((s >> 2) * (L / 16) + f1 * B + l) * 4 + (s & 3);
+}
 __global__ void sympair_kernel(int M, int nsets, int axis, int N, int symstride, int pairstride, const float* sym,
-                               float2* pair);
+                               float2* pair, float* reg);
 __global__ void nonuniform_factor_kernel(int M, int n0, int n1, int n2, size_t tgroup, size_t off1, size_t off2,
                                          int yoff1, int yoff2, const double* nodes, const double* y, double* fac);
 

@@ -175,15 +175,26 @@ __global__ void __launch_bounds__(256) symbol_kernel(int M, int nsets, int glen,
   }
 }
 
-// (s[f], s[N - f]) pairs of one axis for the structured kernels, f < N = L_p/2
+// The symbols of one axis as the structured kernels read them: pairs (s[f], s[N - f]), f < N = L_p/2,
+// and, where the axis has a kernel with its transforms in registers, all L_p values in the order of
+// its threads (symreg_at); the other half of the real symbol of E is its mirror image, that of F the
+// negated one.
 __global__ void sympair_kernel(int M, int nsets, int axis, int N, int symstride, int pairstride, const float* sym,
-                               float2* pair) {
+                               float2* pair, float* reg) {
+  const bool regs = toep_in_registers(N);
   const long total = (long)M * nsets * N;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
     const int f = (int)(i % N);
     const long kt = i / N;  // k * nsets + set
     const float* s = sym + (kt * 3 + axis) * symstride;
     pair[(kt * 3 + axis) * pairstride + f] = make_float2(s[f], s[N - f]);
+    if (regs) {
+      const int set = (int)(kt % nsets);
+      const bool odd = nsets == 2 ? set == 1 : set == axis;
+      float* r = reg + (kt * 3 + axis) * 2 * pairstride;
+      r[symreg_at(f, 2 * N)] = s[f];
+      r[symreg_at(N + f, 2 * N)] = odd ? -s[N - f] : s[N - f];
+    }
   }
 }
 
@@ -365,7 +376,10 @@ extern "C" demag_status demag_build_factors(const demag_grid_desc* d, demag_plan
       dispatch_symbol(P, p, P->M, 2, P->gen64, P->sym, st);
       TRY_CUDA(cudaGetLastError());
     }
-    TRY_CUDA(cudaMalloc(&P->sympair, sizeof(float2) * (size_t)M * 6 * (P->Lmax / 2)));
+    const size_t pairs = (size_t)M * 6 * (P->Lmax / 2);
+    const bool regs = any_toep_in_registers(P);
+    TRY_CUDA(cudaMalloc(&P->sympair, sizeof(float2) * (regs ? 2 : 1) * pairs));
+    if (regs) P->symreg = reinterpret_cast<float*>(P->sympair + pairs);
     for (int p = 0; p < 3; ++p) {
       const int N = P->L[p] / 2;
       const long total = (long)M * 2 * N;
@@ -373,7 +387,7 @@ extern "C" demag_status demag_build_factors(const demag_grid_desc* d, demag_plan
       if (blocks > 152 * 16) blocks = 152 * 16;
       DEMAG_LAUNCH(P, kFamSetup, st,
                    sympair_kernel<<<blocks, 256, 0, st>>>(M, 2, p, N, P->Lmax / 2 + 1, P->Lmax / 2, P->sym,
-                                                          P->sympair));
+                                                          P->sympair, P->symreg));
       TRY_CUDA(cudaGetLastError());
     }
   }

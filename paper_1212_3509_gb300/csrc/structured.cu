@@ -29,6 +29,7 @@
 //                        keep) are computed and stored to HBM.
 // Twiddles: one value per item from a two-level shared table
 // (W_L^m = T1[m >> 7] * T0[m & 127]) and its powers by a product tree.
+#include <algorithm>
 #include <climits>
 #include <type_traits>
 
@@ -63,6 +64,7 @@ struct ToepLaunch {
   int nsets;       // symbol sets per node: 2 (types E, F) or 3 (components of a compressed kernel)
   int diag;        // 1: column (b, q, l) applies node b only and writes it as node 0 of its item
   const float2* sympair;  // [M][nsets][3][pairstride]: (s_f, s_{N-f}); set = type, or q when nsets = 3
+  const float* symreg;    // [M][nsets][3][2 pairstride]: s_f, f < L, in thread order (symreg_at)
 };
 
 template <int LOGN> struct ToepCfg {
@@ -339,6 +341,147 @@ __global__ void __launch_bounds__(256, ToepCfg<LOGN>::minblocks)
     node_loop(std::integral_constant<int, 0>{});
 }
 
+// ---- transforms of 512 to 4096 points in the registers of L / 16 threads
+//
+// Two nodes share one complex transform of length L: a column is real and the
+// symbols of a type are all real (E) or all imaginary (F), so the inverse of
+// (s_k + i s_{k+1}) X is y_k + i y_{k+1}; no split step, no per-column tables.
+// X (times i for F) stays in the registers of its threads for all nodes.
+//
+// f = f1 + 16 f2, t = t0 + 16 B t1 with B = L / 256: the B lanes of group f1
+// transform its 16 B values f2 by one exchange inside their warp (as the 3D
+// passes do), then thread t0 takes its 16 groups from shared memory and does the
+// last 16-point step; the half that is kept is t1 < 8, so only those outputs
+// are computed and a warp's stores are contiguous.  A warp's own rows of the
+// buffer serve the inner exchange before they take its results, and two
+// buffers alternate, so a pair of nodes costs one block barrier.
+//
+// Bound by latency and shared-memory wavefronts (16 warps per SM, held there by
+// 128 registers: X, the values and 16 twiddles twice): per 16 points and pair
+// of nodes 32 wavefronts of symbols and 128 of the two exchanges, where the
+// in-place passes take about 240 per node, four block barriers against one.
+// GB300, R = 61: TT 1024 cells, ranks 8 8, 16 items 338 -> 236 us; CP 1024,
+// r = 4, 64 items 241 -> 150 us; a column's error 2.1e-7 -> 1.3e-7.
+template <int LOGN> struct RegToep {
+  static constexpr int L = 2 << LOGN;
+  static constexpr int B = L / 256;
+  static constexpr int T = L / 16;                  // threads per column
+  static constexpr int THREADS = T < 128 ? 128 : T;
+  static constexpr int G = THREADS / T;             // columns per block
+  static constexpr int BS = RegFft<B>::BS;          // buffer row of one f1
+  static constexpr size_t smem = (size_t)G * 2 * 16 * BS * sizeof(float2);
+  static constexpr int minblocks = 512 / THREADS;   // 16 warps per SM at up to 128 registers
+};
+
+__device__ __forceinline__ float2 ldg_conj(const float2* t) {
+  const float2 w = __ldg(t);
+  return make_float2(w.x, -w.y);
+}
+
+// The twiddles of tw16_idft for w = exp(2 pi i m / L), m < L / 16, from the table exp(-2 pi i m / L).
+__device__ __forceinline__ Twid16 load_twid16(const float2* tab, int m, int L) {
+  Twid16 t;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) t.a[j] = ldg_conj(tab + m + j * (L / 16));
+  t.b[0] = ldg_conj(tab + 2 * m);
+  t.b[1] = ldg_conj(tab + 2 * m + L / 8);
+  t.c = ldg_conj(tab + 4 * m);
+  t.d = ldg_conj(tab + 8 * m);
+  return t;
+}
+
+template <int LOGN>
+__global__ void __launch_bounds__(RegToep<LOGN>::THREADS, RegToep<LOGN>::minblocks)
+    toeplitz_reg_kernel(const __grid_constant__ ToepLaunch a) {
+  using Cfg = RegToep<LOGN>;
+  constexpr int L = Cfg::L, B = Cfg::B, T = Cfg::T, BS = Cfg::BS;
+  extern __shared__ float4 smem_c[];
+  const int g = threadIdx.x / T, lt = threadIdx.x % T;
+  const int f1 = lt / B, l = lt % B;
+  float2* buf = reinterpret_cast<float2*>(smem_c) + (size_t)g * 2 * 16 * BS;
+  const int own = rf_slot<B>(f1) * BS;  // this group's row
+  int slot = 0;
+  while (slot + 1 < a.naxes && (int)blockIdx.x >= a.bx0[slot + 1]) ++slot;
+  const ToepAxis& A = a.ax[slot];
+  const int c = ((int)blockIdx.x - a.bx0[slot]) * Cfg::G + g;
+  const bool active = c < A.ncols;
+  const int rcols = A.rcols, n = A.n, axis = A.axis;
+  const int col = active ? c % rcols : 0, bq = active ? c / rcols : 0;
+  const int q = bq % 3, b = bq / 3;
+  const float* in = A.in + b * A.in_bstride + q * A.in_qstride + (long)col * n;
+
+  // the column's spectrum X in frequency order, once
+  float2 X[16];
+  {
+    float2 x[8], v[16];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) x[r] = make_float2(active && lt + T * r < n ? __ldg(in + lt + T * r) : 0.f, 0.f);
+    dft16_of_half(x, v);
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      buf[rf_slot<B>(k) * BS + lt] = k ? cmul(v[k], __ldg(A.twid + k * lt)) : v[k];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = buf[own + l + B * r];
+    __syncwarp();
+    dft_reg<16, false>(v);
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      buf[own + k * (B + 1) + l] = k ? cmul(v[k], __ldg(A.twid + 16 * k * l)) : v[k];
+    __syncwarp();
+    rf_finish<B>(X, buf + own, l);
+    if (axis == q) {  // F: the symbol is i s
+#pragma unroll
+      for (int s = 0; s < 16; ++s) X[s] = make_float2(-X[s].y, X[s].x);
+    }
+  }
+  const Twid16 tin = load_twid16(A.twid, 16 * l, L), tout = load_twid16(A.twid, lt, L);
+
+  const int set = a.nsets == 3 ? q : (axis == q ? 1 : 0);
+  const int k0 = blockIdx.y * a.kgroup, k1 = min(min(a.M, A.kmax), k0 + a.kgroup);
+  const long kstride = (long)a.nsets * 3 * 2 * a.pairstride;
+  const float4* sp = reinterpret_cast<const float4*>(a.symreg + k0 * kstride + (set * 3 + axis) * 2L * a.pairstride) + lt;
+  const long ostride = 3L * rcols * n;
+  float* out = A.out + b * A.out_bstride + ((long)k0 * 3 + q) * rcols * n + (long)col * n + lt;
+  for (int k = k0; k < k1; k += 2) {
+    const bool two = k + 1 < k1;
+    float2 u[16];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const float4 p = __ldg(sp + s * T);
+      const float4 p2 = two ? __ldg(sp + kstride / 4 + s * T) : make_float4(0.f, 0.f, 0.f, 0.f);
+      u[4 * s + 0] = cmul(X[4 * s + 0], make_float2(p.x, p2.x));
+      u[4 * s + 1] = cmul(X[4 * s + 1], make_float2(p.y, p2.y));
+      u[4 * s + 2] = cmul(X[4 * s + 2], make_float2(p.z, p2.z));
+      u[4 * s + 3] = cmul(X[4 * s + 3], make_float2(p.w, p2.w));
+    }
+    rf_begin<B>(u, buf + own, l);
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 16; ++r) u[r] = buf[own + r * (B + 1) + l];
+    __syncwarp();
+    tw16_idft<16, false>(tin, u);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) buf[own + l + B * r] = u[r];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 16; ++r) u[r] = buf[rf_slot<B>(r) * BS + lt];
+    tw16_idft<16, true>(tout, u);
+    if (active) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        if (lt + T * r < n) {
+          out[T * r] = u[r].x;
+          if (two) out[ostride + T * r] = u[r].y;
+        }
+      }
+    }
+    sp += 2 * (kstride / 4);
+    out += 2 * ostride;
+    buf = reinterpret_cast<float2*>(smem_c) + (size_t)g * 2 * 16 * BS + ((k - k0) & 2 ? 0 : 16 * BS);
+  }
+}
+
 // weights: out_w[b][k][q][l] = c s omega_k * lambda[b][q][l] (lambda NULL -> 1)
 __global__ void weights_kernel(int M, int batch, int rq, const double* scale, const float* lambda,
                                float* out_w) {
@@ -377,19 +520,53 @@ static cudaError_t launch_toep(demag_plan* P, const ToepLaunch& a, int gx, cudaS
   return cudaGetLastError();
 }
 
+template <int LOGN>
+static cudaError_t launch_reg(demag_plan* P, const ToepLaunch& a, int gx, cudaStream_t st) {
+  using Cfg = RegToep<LOGN>;
+  if (Cfg::smem > 48 * 1024) {
+    static unsigned long long done = 0;  // devices whose limit is raised (no attribute calls under capture)
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(done & bit)) {
+      cudaError_t e = cudaFuncSetAttribute(toeplitz_reg_kernel<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)Cfg::smem);
+      if (e != cudaSuccess) return e;
+      done |= bit;
+    }
+  }
+  int gy = (a.M + a.kgroup - 1) / a.kgroup;
+  DEMAG_LAUNCH(P, kFamFFT, st, toeplitz_reg_kernel<LOGN><<<dim3(gx, gy), Cfg::THREADS, Cfg::smem, st>>>(a));
+  return cudaGetLastError();
+}
+
 static int ilog2i(int v) {
   int l = 0;
   while ((1 << l) < v) ++l;
   return l;
 }
 
-static int groups_per_block(int logn) {
+// The register kernel takes every launch of its lengths but the one of a single node per column
+// (the full format's fibres), where half of its paired transform would be empty.
+static bool in_registers(int logn, int diag) { return !diag && toep_in_registers(1 << logn); }
+
+static int groups_per_block(int logn, int diag) {
   int N = 1 << logn;
+  if (in_registers(logn, diag)) return N >= 1024 ? 1 : 1024 / N;
   int TG = N / 16 < 16 ? 16 : (N / 16 > 256 ? 256 : N / 16);
   return 256 / TG;
 }
 
 static cudaError_t launch_logn(demag_plan* P, int logn, const ToepLaunch& a, int gx, cudaStream_t st) {
+  if (in_registers(logn, a.diag)) {
+    switch (logn) {
+      case 8: return launch_reg<8>(P, a, gx, st);
+      case 9: return launch_reg<9>(P, a, gx, st);
+      case 10: return launch_reg<10>(P, a, gx, st);
+      case 11: return launch_reg<11>(P, a, gx, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   switch (logn) {
     case 0: return launch_toep<0>(P, a, gx, st);
     case 1: return launch_toep<1>(P, a, gx, st);
@@ -409,28 +586,37 @@ static cudaError_t launch_logn(demag_plan* P, int logn, const ToepLaunch& a, int
   }
 }
 
-// Nodes per block.  Each block transforms its columns once and reuses the
+// Nodes per block (an even number, or all, in the register kernel).  Each block transforms its columns once and reuses the
 // spectra for kgroup nodes, so large groups save forward FFTs, while small
 // groups give more blocks.  Default: the largest group that still yields
-// eight blocks per SM; with autotuning on, the candidates M, M/2, M/4, ..., 1
+// eight blocks per SM; in the register kernel, where a forward transform costs
+// as much as two nodes, half of the blocks that are resident at once (CP 2048,
+// r = 4, 8 items 105 -> 55 us, TT 700, ranks 3 5, 3 items 30 -> 20 us; all of
+// the resident ones 62 and 22 us, and CP 400, 4 items 14 against 17 us); with autotuning on, the candidates M, M/2, M/4, ..., 1
 // are timed once per (FFT length, column blocks, M) and the fastest is kept.
 static cudaError_t pick_kgroup(demag_plan* P, int logn, ToepLaunch& a, int gx, cudaStream_t st) {
   const int M = a.M;
+  // nodes go in pairs in the register kernel: groups of an even number, or all nodes, so that the
+  // pairs and with them the results do not depend on the group
+  const bool paired = in_registers(logn, a.diag);
+  auto rounded = [&](int c) { return paired ? std::min(c + (c & 1), M) : c; };
   for (const demag_plan::Tuned& t : P->tuned)
     if (t.kind == 0 && t.key[0] == logn && t.key[1] == gx && t.key[2] == M) {
-      a.kgroup = t.value;
+      a.kgroup = rounded(t.value);
       return cudaSuccess;
     }
+  const int least = paired ? 2 : 1;
+  const long enough = !paired ? 1216 : logn == 11 ? 152 : 304;
   int kg = M;
-  while (kg > 1 && (long)gx * ((M + kg - 1) / kg) < 1216) kg = (kg + 1) / 2;
+  while (kg > least && (long)gx * ((M + kg - 1) / kg) < enough) kg = rounded((kg + 1) / 2);
   a.kgroup = kg;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(st, &cap);
   if (!P->autotune || cap != cudaStreamCaptureStatusNone) return cudaSuccess;
   std::vector<int> cands;
-  for (int c = M;; c = (c + 1) / 2) {
+  for (int c = M;; c = rounded((c + 1) / 2)) {
     if (cands.empty() || cands.back() != c) cands.push_back(c);
-    if (c == 1) break;
+    if (c <= least) break;
   }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -473,16 +659,19 @@ static cudaError_t pick_kgroup(demag_plan* P, int logn, ToepLaunch& a, int gx, c
 // Toeplitz matvecs of the given axes: axes that share an FFT length run in
 // one launch (normally all three), each as its own range of blocks.
 static demag_status run_axes(demag_plan* P, ToepAxis* axes, int count, const char* what, cudaStream_t st,
-                             const float2* sympair = nullptr, int nsets = 2, int diag = 0) {
+                             const float2* sympair = nullptr, const float* symreg = nullptr, int nsets = 2,
+                             int diag = 0) {
   bool done[3] = {false, false, false};
   for (int i = 0; i < count; ++i) {
     if (done[i]) continue;
     const int logn = ilog2i(P->L[axes[i].axis] / 2);
-    const int G = groups_per_block(logn);
+    const int G = groups_per_block(logn, diag);
     ToepLaunch a{};
     a.M = 0;
     a.pairstride = P->Lmax / 2;
     a.sympair = sympair ? sympair : P->sympair;
+    a.symreg = symreg ? symreg : P->symreg;
+    a.diag = diag;
     a.nsets = nsets;
     int gx = 0;
     for (int j = i; j < count; ++j) {
@@ -499,7 +688,6 @@ static demag_status run_axes(demag_plan* P, ToepAxis* axes, int count, const cha
       done[j] = true;
     }
     a.bx0[a.naxes] = gx;
-    a.diag = diag;
     cudaError_t e = cudaSuccess;
     if (diag)
       a.kgroup = a.M;  // one node per column: grid.y = 1
@@ -645,7 +833,7 @@ extern "C" demag_status demag_apply_full_fibres(demag_plan* P, const float* m, f
   b.in_qstride = N;
   b.out = Y;
   b.out_bstride = 3 * N;
-  s = run_axes(P, &b, 1, "toeplitz_fft_kernel (fibres, axis 2)", st, nullptr, 2, 1);
+  s = run_axes(P, &b, 1, "toeplitz_fft_kernel (fibres, axis 2)", st, nullptr, nullptr, 2, 1);
   if (s != DEMAG_OK) return s;
   // Z[k][q][i1][i2][i3]
   {
@@ -665,7 +853,7 @@ extern "C" demag_status demag_apply_full_fibres(demag_plan* P, const float* m, f
   c.in_qstride = N;
   c.out = Y;
   c.out_bstride = 3 * N;
-  s = run_axes(P, &c, 1, "toeplitz_fft_kernel (fibres, axis 3)", st, nullptr, 2, 1);
+  s = run_axes(P, &c, 1, "toeplitz_fft_kernel (fibres, axis 3)", st, nullptr, nullptr, 2, 1);
   if (s != DEMAG_OK) return s;
   {
     const long tiles = (long)n2 * ((n1 + 31) / 32) * ((n3 + 31) / 32);
@@ -778,7 +966,7 @@ extern "C" demag_status demag_apply_tucker_compressed(demag_plan* P, int batch, 
     aoff += (long)r[p] * P->n[p];
     ooff += 3L * cv.rho[p] * r[p] * P->n[p];
   }
-  s = run_axes(P, ax, 3, "toeplitz_fft_kernel (compressed tucker)", st, cv.cpair, 3);
+  s = run_axes(P, ax, 3, "toeplitz_fft_kernel (compressed tucker)", st, cv.cpair, cv.creg, 3);
   if (s != DEMAG_OK || !out_core) return s;
   return launch_core_kron(P, batch, r, core, out_core, st);
 }
