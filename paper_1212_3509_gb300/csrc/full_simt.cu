@@ -21,6 +21,7 @@
 // while a tile is loaded and y_a = p_a + q_a, y_{n-1-a} = p_a - q_a in its
 // epilogue: no folded copy of any field exists.  A factor without that
 // symmetry (non-uniform grid) is the sum of two such parts.
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cooperative_groups.h>
@@ -608,17 +609,37 @@ static cudaError_t launch_mode_cfg(demag_plan* P, ModeStage S, int split, cudaSt
 // 129, split over 4 blocks 45, 64 x 16 over 8 blocks 26.5.
 struct ModeShape {
   int bm, bn, occ;
-  double rate;
+  double rate, fill;  // at full occupancy; exponent of the resident share below it
 };
+
+//
+// A split sum runs as clusters, and three things decide its time beside that:
+// the longest node range (20 nodes over 6 or 7 blocks: 4 and 3); the share of the
+// block slots that clusters of one size can fill (as
+// cudaOccupancyMaxActiveClusters reports it: 266 of 304 for 7 blocks, 296 for 4);
+// and, when there are few, that a cluster stays in one of eight groups of up to
+// 20 SMs, which 3 clusters of 7 overfill while others idle.  With them, and its
+// own rates, the sum's choice is 0.3% off the fastest split and tile on average
+// over 14 FP32 grids (1.3% at most), where the model of whole SMs was 6% (18%)
+// off: 128^3 1170 -> 1130 us, 112^3 823 -> 748, 64^3 146 -> 124, 128 x 40 x 60
+// 220 -> 188 (the whole application).
+static double cluster_share(int occ, int split) {
+  static const double share[3][9] = {{1, 1, 1, .957, .974, .954, .908, .875, .947},   // 2 blocks per SM
+                                     {1, 1, 1, .974, .965, .954, .974, .906, .895},   // 3
+                                     {1, 1, 1, .970, .974, .966, .957, .938, .974}};  // 6 or 8
+  return share[occ <= 2 ? 0 : occ <= 3 ? 1 : 2][split];
+}
 
 static double mode_cost(const ModeStage& S, bool sum, const ModeShape& c, int split) {
   double pairs = 0;
   for (int j = 0; j < S.njobs; ++j) pairs += S.npairs[j];
   pairs /= S.njobs;
   const double tiles = std::ceil((double)S.rows / c.bm) * ((S.h + c.bn - 1) / c.bn) * S.njobs * (sum ? split : S.nodes);
-  const double steps = (double)((S.h + kBK - 1) / kBK * kBK) * pairs * (sum ? (double)S.nodes / split : 1.0);
-  const double per_sm = std::ceil(tiles / 152.0);
-  const double full = per_sm < c.occ ? std::pow(per_sm / c.occ, 0.3) : 1.0;
+  const double steps = (double)((S.h + kBK - 1) / kBK * kBK) * pairs *
+                       (sum ? 0.8 * ((S.nodes + split - 1) / split) + 0.2 * S.nodes / split : 1.0);
+  double per_sm = std::ceil(tiles / (152.0 * cluster_share(c.occ, split)) - 1e-9);
+  if (split > 1) per_sm = std::max(per_sm, std::ceil(std::ceil(tiles / split / 8) * split / 20));
+  const double full = per_sm < c.occ ? std::pow(per_sm / c.occ, c.fill) : 1.0;
   return per_sm * (steps + 24 + (split > 1 ? 48 : 0)) * c.bm * c.bn / (c.rate * full);
 }
 
@@ -633,20 +654,21 @@ static cudaError_t launch_mode(demag_plan* P, const ModeStage& S, cudaStream_t s
   int count = 0;
   auto add = [&](auto cfg, double rate) {
     using Cfg = decltype(cfg);
-    all[count++] = {{Cfg::BM, Cfg::BN, Cfg::OCC, rate}, launch_mode_cfg<T, Cfg, KIND>};
+    all[count++] = {{Cfg::BM, Cfg::BN, Cfg::OCC, rate, SUM && std::is_same<T, float>::value ? 0.7 : 0.3},
+                    launch_mode_cfg<T, Cfg, KIND>};
   };
   if constexpr (std::is_same<T, float>::value) {
     add(ModeCfg<float, 128, 64, 8, 8, 2>{}, 1.0);
     add(ModeCfg<float, 256, 32, 8, 8, 2>{}, 0.95);
-    add(ModeCfg<float, 128, 32, 8, 4, 3>{}, 0.8);
-    add(ModeCfg<float, 256, 16, 8, 4, 3>{}, 0.8);
+    add(ModeCfg<float, 128, 32, 8, 4, 3>{}, SUM ? 0.85 : 0.8);
+    add(ModeCfg<float, 256, 16, 8, 4, 3>{}, SUM ? 0.85 : 0.8);
     add(ModeCfg<float, 64, 16, 4, 2, 8>{}, 0.6);
   } else {
     // FP64 multiply-adds run at 1/64 of the FP32 rate: any tile feeds them, and small ones balance the SMs
     add(ModeCfg<double, 64, 32, 4, 4, 3>{}, 1.0);
     add(ModeCfg<double, 32, 16, 2, 2, 6>{}, 0.9);
   }
-  const int most = SUM ? (S.nodes < 8 ? S.nodes : 8) : 1;
+  const int most = SUM ? std::min(S.nodes, 8) : 1;
   const Choice* pick = nullptr;
   int split = 1;
   double best = 0;
@@ -659,6 +681,12 @@ static cudaError_t launch_mode(demag_plan* P, const ModeStage& S, cudaStream_t s
         split = s;
       }
     }
+  // an FP32 sum goes to four blocks where the model sees little between them and fewer: shorter chains of
+  // additions (128^3: error 5.7e-7 over 2 blocks, 3.0e-7 over 4, 1130 and 1127 us); where they fill the
+  // chip worse they stay fewer (200 x 64 x 150: 1360 us against 1542)
+  if (SUM && std::is_same<T, float>::value && split < 4 && most >= 4 &&
+      mode_cost(S, true, pick->shape, 4) <= 1.06 * best)
+    split = 4;
   return pick->run(P, S, split, st);
 }
 
