@@ -2206,6 +2206,11 @@ static void set_stage(TcGroup& G, const CUtensorMap& ahi, const CUtensorMap& alo
   G.n_tiles = (n_a + bn - 1) / bn;
 }
 
+// Whether tiles of `bn` columns may go out through TMA: the epilogue stores whole boxes of 32 columns,
+// clipped at the end of the half and not at the end of a tile, so a tile that has a neighbour must be a
+// multiple of 32 wide (its last box would otherwise overwrite the neighbour's first columns).
+static bool tile_width_fits(const TcGroup& G, int bn) { return !G.tma_out || bn >= G.n_a || bn % 32 == 0; }
+
 static demag_status build_programs(demag_plan* P, TcState* S, const CUtensorMap (&mapX)[2],
                                    const CUtensorMap (&map1)[2], const CUtensorMap (&map2)[2],
                                    const CUtensorMap (&mapB)[3][2], const CUtensorMap (&out1)[2],
@@ -2309,6 +2314,7 @@ static demag_status build_programs(demag_plan* P, TcState* S, const CUtensorMap 
       if (stage == 0) { H[p].o_hi = out1[0]; H[p].o_lo = out1[1]; H[p].w_hi = wout1[0]; H[p].w_lo = wout1[1]; }
       if (stage == 1) { H[p].o_hi = out2[0]; H[p].o_lo = out2[1]; H[p].w_hi = wout2[0]; H[p].w_lo = wout2[1]; }
       if (stage == 2) { H[p].o_hi = out3; H[p].w_hi = wout3; }
+      if (!tile_width_fits(H[p], H[p].bn)) H[p].tma_out = 0;  // plain stores stop at the tile's own columns
     }
   }
   // job and pair tables
@@ -2420,6 +2426,7 @@ static demag_status set_tile_width(demag_plan* P, TcState* S, int prog, int bn) 
   TcGroup& G = S->host_prog[prog];
   const int axis = prog_axis(prog);
   const int M = P->M;
+  if (!tile_width_fits(G, bn)) return set_error(P, DEMAG_EINVAL, "tile width %d does not divide into store boxes", bn);
   for (int h = 0; h < 2; ++h)
     if (!make_bmap(h ? &G.b_lo : &G.b_hi, S->B[axis][h], S->elem, S->geo.h[axis], S->halves[axis], 2 * M,
                    S->ldB[axis], bn))
@@ -2477,7 +2484,9 @@ static demag_status apply_tuned(demag_plan* P, TcState* S) {
     for (int knob = 0; knob < 4; ++knob) {
       const demag_plan::Tuned* t = find_tuned(P, tune_kind(S, knob), prog);
       if (!t) continue;
-      if (knob == 0 && !(t->value >= 16 && t->value <= kBN && t->value % 16 == 0)) continue;
+      if (knob == 0 && !(t->value >= 16 && t->value <= kBN && t->value % 16 == 0 &&
+                         tile_width_fits(S->host_prog[prog], t->value)))
+        continue;
       demag_status s = set_knob(P, S, prog, knob, t->value);
       if (s != DEMAG_OK) return s;
     }
@@ -3168,7 +3177,7 @@ demag_status tc_batch_create(demag_plan* const* plans, int count, demag_precisio
           const TcState* S = state(plans[order[i]], prec);
           const int axis = B->fused[order[i]] && st3 == 0 ? 2 : st3;
           const int tiles = (G.n_a + 127) / 128;
-          G.bn = round_up((G.n_a + tiles - 1) / tiles, 16);
+          G.bn = round_up((G.n_a + tiles - 1) / tiles, 32);  // at most 128, and whole store boxes (tile_width_fits)
           G.n_tiles = (G.n_a + G.bn - 1) / G.bn;
           G.ntiles = G.njobs * G.m_tiles * G.n_tiles;
           for (int h = 0; h < 2; ++h)
