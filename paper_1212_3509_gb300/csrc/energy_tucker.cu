@@ -23,9 +23,7 @@
 namespace demag {
 
 constexpr int kEnMaxRank = 64;
-// static shared memory of the energy kernels: the partial sums of block_gram and a reduction buffer
 constexpr int kEnWarps = 8;
-constexpr size_t kEnStaticSmem = (kEnWarps * 64 + 32) * sizeof(double);
 constexpr size_t kEnSmemMax = 200 * 1024;  // largest dynamic request (Grams, and the contraction where it fits)
 
 __device__ __forceinline__ double en_warp_sum(double v) {
@@ -109,6 +107,15 @@ struct EnGram {
   bool deriv;
   double scale;
   double* M;
+};
+
+// Static shared memory of the energy kernels; its size counts against the 48 KB that a launch may ask
+// for without the attribute.
+template <typename F>
+struct EnShared {
+  double red[32];             // the block's sum
+  double part[kEnWarps * 64]; // partial Gram blocks of block_grams
+  EnGram<F> gram[3];
 };
 
 // The three Grams g[0..2] (in shared memory) by the whole block.  The work is cut into items, 8 x 8
@@ -215,8 +222,9 @@ __device__ void block_grams(const EnGram<F>* g, double* part) {
 template <typename F>
 __global__ void __launch_bounds__(32 * kEnWarps) tucker_energy_kernel(const __grid_constant__ EnTuckerT<F> a) {
   extern __shared__ double Mg[];
-  __shared__ double red[32], gpart[kEnWarps * 64];
-  __shared__ EnGram<F> gram[3];
+  __shared__ EnShared<F> sh;
+  double* const red = sh.red;
+  EnGram<F>* const gram = sh.gram;
   const int t = blockIdx.x, q = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int r1 = a.r[0], r2 = a.r[1], r3 = a.r[2];
@@ -237,7 +245,7 @@ __global__ void __launch_bounds__(32 * kEnWarps) tucker_energy_kernel(const __gr
   if (Cd)
     for (int i = threadIdx.x; i < size_c; i += blockDim.x) Cd[i] = (double)Ct[i];
   __syncthreads();
-  block_grams(gram, gpart);
+  block_grams(gram, sh.part);
   const double *M1 = Mg, *M2 = Mg + moff[1], *M3 = Mg + moff[2];
   double* Y1 = a.ws ? a.ws + ((long)t * 3 + q) * ((long)r1 * s3 * (s2 + r2)) : Cd + size_c;
   double* Y2 = Y1 + r1 * s2 * s3;
@@ -299,8 +307,9 @@ struct EnTT {
 
 __global__ void __launch_bounds__(32 * kEnWarps) tt_energy_kernel(const __grid_constant__ EnTT a) {
   extern __shared__ double sg[];
-  __shared__ double red[32], gpart[kEnWarps * 64];
-  __shared__ EnGram<float> gram[3];
+  __shared__ EnShared<float> sh;
+  double* const red = sh.red;
+  EnGram<float>* const gram = sh.gram;
   const int t = blockIdx.x, q = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int r1 = a.r1, r2 = a.r2, r12 = r1 * r2;
@@ -310,7 +319,7 @@ __global__ void __launch_bounds__(32 * kEnWarps) tt_energy_kernel(const __grid_c
     gram[p] = {a.A[p] + (long)q * rp * n, a.B[p] + (long)t * rp * n, rp, rp, n, p == q, a.inv2h[p], Mg[p]};
   }
   __syncthreads();
-  block_grams(gram, gpart);
+  block_grams(gram, sh.part);
   double x = 0.0;
   for (int e = threadIdx.x; e < r2 * r2; e += blockDim.x) {
     const int a2 = e / r2, b2 = e % r2;
@@ -395,7 +404,7 @@ static demag_status run_tucker_energy(demag_plan* P, EnTuckerT<F>& a, double* en
   const long per = (long)a.r[0] * a.s[2] * (a.s[1] + a.r[1]), core = (long)a.s[0] * a.s[1] * a.s[2];
   const bool in_smem = sizeof(double) * (grams + per + core) <= 96 * 1024;
   const size_t smem = sizeof(double) * (grams + (in_smem ? per + core : 0));
-  if (smem + kEnStaticSmem > 48 * 1024) {
+  if (smem + sizeof(EnShared<F>) > 48 * 1024) {
     static unsigned long long done = 0;  // one per instantiation
     int dev = 0;
     cudaGetDevice(&dev);
@@ -511,7 +520,7 @@ extern "C" demag_status demag_energy_tt(demag_plan* P, const int r[2], const flo
   a.T = 3 * P->M;
   const int r12 = r[0] * r[1];
   const size_t smem = sizeof(double) * ((size_t)r[0] * r[0] + (size_t)r12 * r12 + (size_t)r[1] * r[1]);
-  if (smem + kEnStaticSmem > 48 * 1024) {  // dynamic plus the kernels' static tiles
+  if (smem + sizeof(EnShared<float>) > 48 * 1024) {
     static unsigned long long done = 0;
     int dev = 0;
     cudaGetDevice(&dev);
