@@ -41,7 +41,7 @@ struct Compressed {
   double* cgen = nullptr;   // [rhomax][3 q][3 p][glen] compressed generators
   float* csym = nullptr;    // [rhomax][3][3][Lmax/2 + 1]
   float2* cpair = nullptr;  // [rhomax][3][3][Lmax/2]
-  float* creg = nullptr;    // [rhomax][3][3][Lmax] in thread order (symreg_at), behind cpair
+  float* creg = nullptr;    // [rhomax][3][3][regstride] in thread order (symreg_kernel), behind cpair
   float* core = nullptr;    // [3 q][rho3][rho2][rho1]
 };
 
@@ -890,9 +890,8 @@ extern "C" demag_status demag_compress_kernel(demag_plan* P, double tol, void* s
   CMP_CUDA(cudaMalloc(&C->csym, sizeof(float) * (size_t)rmax * 9 * symstride));
   CMP_CUDA(cudaMemsetAsync(C->csym, 0, sizeof(float) * (size_t)rmax * 9 * symstride, st));
   const size_t pairs = (size_t)rmax * 9 * pairstride;
-  const bool regs = any_toep_in_registers(P);
-  CMP_CUDA(cudaMalloc(&C->cpair, sizeof(float2) * (regs ? 2 : 1) * pairs));
-  if (regs) C->creg = reinterpret_cast<float*>(C->cpair + pairs);
+  CMP_CUDA(cudaMalloc(&C->cpair, sizeof(float2) * pairs + sizeof(float) * (size_t)rmax * 9 * P->regstride));
+  if (P->regstride) C->creg = reinterpret_cast<float*>(C->cpair + pairs);
   for (int p = 0; p < 3; ++p) {
     dispatch_symbol(P, p, C->rho[p], 3, C->cgen, C->csym, st);
     CMP_CUDA(cudaGetLastError());
@@ -902,7 +901,11 @@ extern "C" demag_status demag_compress_kernel(demag_plan* P, double tol, void* s
     if (blocks > 152 * 16) blocks = 152 * 16;
     DEMAG_LAUNCH(P, kFamSetup, st,
                  sympair_kernel<<<(int)blocks, 256, 0, st>>>(C->rho[p], 3, p, N, symstride, pairstride, C->csym,
-                                                             C->cpair, C->creg));
+                                                             C->cpair));
+    CMP_CUDA(cudaGetLastError());
+    if (!toep_in_registers(N)) continue;
+    DEMAG_LAUNCH(P, kFamSetup, st,
+                 symreg_kernel<<<3 * C->rho[p], 256, 0, st>>>(3, p, N, symstride, P->regstride, C->csym, C->creg));
     CMP_CUDA(cudaGetLastError());
   }
   CMP_CUDA(cudaStreamSynchronize(st));

@@ -49,7 +49,9 @@ struct demag_plan {
   float* sym = nullptr;      // [M][2][3][Lmax/2 + 1] symbols / L_p
   float2* twid[3] = {nullptr, nullptr, nullptr};  // per axis: exp(-2 pi i m / L_p), m < L_p
   float2* sympair = nullptr; // [M][2][3][Lmax/2]: (symbol[f], symbol[L_p/2 - f]) for f < L_p/2
-  float* symreg = nullptr;   // [M][2][3][Lmax]: all L_p symbol values in thread order (symreg_at), behind sympair
+  float* symreg = nullptr;   // [M][2][3][regstride]: all L_p symbol values in thread order (symreg_at), times a
+                             // power of two, and its reciprocal (symreg_kernel), behind sympair
+  int regstride = 0;
   double* scale = nullptr;   // [M]: c * s * omega_k
   double* gend = nullptr;    // [M][2][3][glen]: derivative generators dE/s, dF/s (lazily, analytic stray field)
 
@@ -188,7 +190,7 @@ void tc_destroy(demag_plan* plan);
 struct CompressedView {
   int rho[3];
   const float2* cpair;  // symbol pairs [rhomax][3 q][3 p][Lmax/2]
-  const float* creg;    // all symbol values in thread order [rhomax][3 q][3 p][Lmax]
+  const float* creg;    // all symbol values in thread order, as symreg [rhomax][3 q][3 p][regstride]
   const float* core;    // [3 q][rho3][rho2][rho1]
 };
 bool compressed_view(const demag_plan* plan, CompressedView* v);
@@ -225,7 +227,8 @@ __host__ __device__ inline int symreg_at(int f, int L) {
   return ((s >> 2) * (L / 16) + f1 * B + l) * 4 + (s & 3);
 }
 __global__ void sympair_kernel(int M, int nsets, int axis, int N, int symstride, int pairstride, const float* sym,
-                               float2* pair, float* reg);
+                               float2* pair);
+__global__ void symreg_kernel(int nsets, int axis, int N, int symstride, int regstride, const float* sym, float* reg);
 __global__ void nonuniform_factor_kernel(int M, int n0, int n1, int n2, size_t tgroup, size_t off1, size_t off2,
                                          int yoff1, int yoff2, const double* nodes, const double* y, double* fac);
 

@@ -175,27 +175,60 @@ __global__ void __launch_bounds__(256) symbol_kernel(int M, int nsets, int glen,
   }
 }
 
-// The symbols of one axis as the structured kernels read them: pairs (s[f], s[N - f]), f < N = L_p/2,
-// and, where the axis has a kernel with its transforms in registers, all L_p values in the order of
-// its threads (symreg_at); the other half of the real symbol of E is its mirror image, that of F the
-// negated one.
+// (s[f], s[N - f]) pairs of one axis for the structured kernels, f < N = L_p/2
 __global__ void sympair_kernel(int M, int nsets, int axis, int N, int symstride, int pairstride, const float* sym,
-                               float2* pair, float* reg) {
-  const bool regs = toep_in_registers(N);
+                               float2* pair) {
   const long total = (long)M * nsets * N;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
     const int f = (int)(i % N);
     const long kt = i / N;  // k * nsets + set
     const float* s = sym + (kt * 3 + axis) * symstride;
     pair[(kt * 3 + axis) * pairstride + f] = make_float2(s[f], s[N - f]);
-    if (regs) {
-      const int set = (int)(kt % nsets);
-      const bool odd = nsets == 2 ? set == 1 : set == axis;
-      float* r = reg + (kt * 3 + axis) * 2 * pairstride;
-      r[symreg_at(f, 2 * N)] = s[f];
-      r[symreg_at(N + f, 2 * N)] = odd ? -s[N - f] : s[N - f];
-    }
   }
+}
+
+// The same symbols for the kernel with its transforms in registers, one block per node and set: all
+// L_p = 2 N values in the order of its threads (symreg_at); the second half of the real symbol of E
+// is its mirror image, that of F the negated one.  Nodes 2 j and 2 j + 1 share a complex transform there,
+// whose rounding errors are relative to the larger of them, and neighbours may differ by orders of
+// magnitude (F of 129 cells, R = 61: the last two nodes 40 : 1).  So the odd one is brought to the
+// Euclidean norm of the even one by a power of two, exact in both directions, whose reciprocal stands
+// behind its L_p values.
+__global__ void __launch_bounds__(256) symreg_kernel(int nsets, int axis, int N, int symstride, int regstride,
+                                                     const float* sym, float* reg) {
+  __shared__ double sum[2][256];
+  const int kt = blockIdx.x;  // k * nsets + set
+  const int set = kt % nsets;
+  const bool odd = nsets == 2 ? set == 1 : set == axis;
+  const bool second = (kt / nsets) % 2 == 1;
+  const float* s = sym + ((long)kt * 3 + axis) * symstride;
+  const float* s0 = second ? s - (long)nsets * 3 * symstride : s;
+  double v = 0.0, v0 = 0.0;
+  for (int f = threadIdx.x; f < N; f += 256) {
+    v += (double)s[f] * s[f] + (double)s[N - f] * s[N - f];
+    v0 += (double)s0[f] * s0[f] + (double)s0[N - f] * s0[N - f];
+  }
+  sum[0][threadIdx.x] = v;
+  sum[1][threadIdx.x] = v0;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) {
+      sum[0][threadIdx.x] += sum[0][threadIdx.x + o];
+      sum[1][threadIdx.x] += sum[1][threadIdx.x + o];
+    }
+    __syncthreads();
+  }
+  v = sum[0][0];
+  v0 = sum[1][0];
+  const int e = v > 0.0 && v0 > 0.0 ? max(-120, min(120, (int)rint(0.5 * (log2(v0) - log2(v))))) : 0;
+  const float up = ldexpf(1.f, e);
+  float* r = reg + ((long)kt * 3 + axis) * regstride;
+  for (int f = threadIdx.x; f < N; f += 256) {
+    const float a = up * s[f], b = up * s[N - f];
+    r[symreg_at(f, 2 * N)] = a;
+    r[symreg_at(N + f, 2 * N)] = odd ? -b : b;
+  }
+  if (threadIdx.x == 0) r[2 * N] = ldexpf(1.f, -e);
 }
 
 __global__ void twiddle_kernel(int L, float2* tw) {
@@ -378,7 +411,8 @@ extern "C" demag_status demag_build_factors(const demag_grid_desc* d, demag_plan
     }
     const size_t pairs = (size_t)M * 6 * (P->Lmax / 2);
     const bool regs = any_toep_in_registers(P);
-    TRY_CUDA(cudaMalloc(&P->sympair, sizeof(float2) * (regs ? 2 : 1) * pairs));
+    P->regstride = regs ? P->Lmax + 32 : 0;  // 128-byte rows: a warp loads 512 bytes at once
+    TRY_CUDA(cudaMalloc(&P->sympair, sizeof(float2) * pairs + sizeof(float) * (size_t)M * 6 * P->regstride));
     if (regs) P->symreg = reinterpret_cast<float*>(P->sympair + pairs);
     for (int p = 0; p < 3; ++p) {
       const int N = P->L[p] / 2;
@@ -387,7 +421,11 @@ extern "C" demag_status demag_build_factors(const demag_grid_desc* d, demag_plan
       if (blocks > 152 * 16) blocks = 152 * 16;
       DEMAG_LAUNCH(P, kFamSetup, st,
                    sympair_kernel<<<blocks, 256, 0, st>>>(M, 2, p, N, P->Lmax / 2 + 1, P->Lmax / 2, P->sym,
-                                                          P->sympair, P->symreg));
+                                                          P->sympair));
+      TRY_CUDA(cudaGetLastError());
+      if (!toep_in_registers(N)) continue;
+      DEMAG_LAUNCH(P, kFamSetup, st,
+                   symreg_kernel<<<2 * M, 256, 0, st>>>(2, p, N, P->Lmax / 2 + 1, P->regstride, P->sym, P->symreg));
       TRY_CUDA(cudaGetLastError());
     }
   }

@@ -67,7 +67,9 @@ struct ToepLaunch {
   int nsets;       // symbol sets per node: 2 (types E, F) or 3 (components of a compressed kernel)
   int diag;        // 1: column (b, q, l) applies node b only and writes it as node 0 of its item
   const float2* sympair;  // [M][nsets][3][pairstride]: (s_f, s_{N-f}); set = type, or q when nsets = 3
-  const float* symreg;    // [M][nsets][3][2 pairstride]: s_f, f < L, in thread order (symreg_at)
+  const float* symreg;    // [M][nsets][3][regstride]: s_f, f < L, in thread order, scaled, and what takes the
+                          // outputs back (symreg_kernel)
+  int regstride;
 };
 
 template <int LOGN> struct ToepCfg {
@@ -349,7 +351,11 @@ __global__ void __launch_bounds__(256, ToepCfg<LOGN>::minblocks)
 // Two nodes share one complex transform of length L: a column is real and the
 // symbols of a type are all real (E) or all imaginary (F), so the inverse of
 // (s_k + i s_{k+1}) X is y_k + i y_{k+1}; no split step, no per-column tables.
-// X (times i for F) stays in the registers of its threads for all nodes.
+// X (times i for F) stays in the registers of its threads for all nodes.  The
+// odd node's symbols carry a power of two that brings them to the size of the
+// even one's (symreg_kernel), which the store takes back: without it a small
+// node next to a large one loses digits (129 cells, R = 61, F of the last node
+// on constant columns: off by 1.7e-5 of its own norm; 9.6e-7 with it).
 //
 // f = f1 + 16 f2, t = t0 + 16 B t1 with B = L / 256: the B lanes of group f1
 // transform its 16 B values f2 by one exchange inside their warp (as the 3D
@@ -364,8 +370,8 @@ __global__ void __launch_bounds__(256, ToepCfg<LOGN>::minblocks)
 // sets of 8 twiddles): per 16 points and pair
 // of nodes 32 wavefronts of symbols and 128 of the two exchanges, where the
 // in-place passes take about 240 per node, four block barriers against one.
-// GB300, R = 61: TT 1024 cells, ranks 8 8, 16 items 338 -> 237 us; CP 1024,
-// r = 4, 64 items 241 -> 150 us; a column's error 2.1e-7 -> 1.3e-7.  Five blocks
+// GB300, R = 61: TT 1024 cells, ranks 8 8, 16 items 338 -> 238 us; CP 1024,
+// r = 4, 64 items 241 -> 152 us; a column's error 2.1e-7 -> 1.3e-7.  Five blocks
 // of 128 threads per SM (96 registers, spills) 284 us; the next symbols
 // prefetched into L1 156 instead of 150 us for that CP batch.
 template <int LOGN> struct RegToep {
@@ -416,6 +422,12 @@ __global__ void __launch_bounds__(RegToep<LOGN>::THREADS, RegToep<LOGN>::minbloc
   const int q = bq % 3, b = bq / 3;
   const float* in = A.in + b * A.in_bstride + q * A.in_qstride + (long)col * n;
 
+  const int set = a.nsets == 3 ? q : (axis == q ? 1 : 0);
+  const int k0 = blockIdx.y * a.kgroup, k1 = min(min(a.M, A.kmax), k0 + a.kgroup);
+  const long kstride = (long)a.nsets * 3 * a.regstride;
+  const float* row = a.symreg + k0 * kstride + (set * 3 + axis) * (long)a.regstride;
+  const float* back = row + kstride + L;  // what takes the outputs of the odd nodes back from their scaled symbols
+
   // the column's spectrum X in frequency order, once
   float2 X[16];
   {
@@ -443,10 +455,7 @@ __global__ void __launch_bounds__(RegToep<LOGN>::THREADS, RegToep<LOGN>::minbloc
   }
   const Twid16 tin = load_twid16(A.twid, 16 * l, L), tout = load_twid16(A.twid, lt, L);
 
-  const int set = a.nsets == 3 ? q : (axis == q ? 1 : 0);
-  const int k0 = blockIdx.y * a.kgroup, k1 = min(min(a.M, A.kmax), k0 + a.kgroup);
-  const long kstride = (long)a.nsets * 3 * 2 * a.pairstride;
-  const float4* sp = reinterpret_cast<const float4*>(a.symreg + k0 * kstride + (set * 3 + axis) * 2L * a.pairstride) + lt;
+  const float4* sp = reinterpret_cast<const float4*>(row) + lt;
   const long ostride = 3L * rcols * n;
   float* out = A.out + b * A.out_bstride + ((long)k0 * 3 + q) * rcols * n + (long)col * n + lt;
   for (int k = k0; k < k1; k += 2) {
@@ -461,6 +470,7 @@ __global__ void __launch_bounds__(RegToep<LOGN>::THREADS, RegToep<LOGN>::minbloc
       u[4 * s + 2] = cmul(X[4 * s + 2], make_float2(p.z, p2.z));
       u[4 * s + 3] = cmul(X[4 * s + 3], make_float2(p.w, p2.w));
     }
+    const float c = two ? __ldg(back) : 0.f;
     rf_begin<B>(u, buf + own, l);
     __syncwarp();
 #pragma unroll
@@ -478,11 +488,12 @@ __global__ void __launch_bounds__(RegToep<LOGN>::THREADS, RegToep<LOGN>::minbloc
       for (int r = 0; r < 8; ++r) {
         if (lt + T * r < n) {
           out[T * r] = u[r].x;
-          if (two) out[ostride + T * r] = u[r].y;
+          if (two) out[ostride + T * r] = c * u[r].y;
         }
       }
     }
     sp += 2 * (kstride / 4);
+    back += 2 * kstride;
     out += 2 * ostride;
     buf = reinterpret_cast<float2*>(smem_c) + (size_t)g * 2 * 16 * BS + ((k - k0) & 2 ? 0 : 16 * BS);
   }
@@ -665,8 +676,7 @@ static cudaError_t pick_kgroup(demag_plan* P, int logn, ToepLaunch& a, int gx, c
 // Toeplitz matvecs of the given axes: axes that share an FFT length run in
 // one launch (normally all three), each as its own range of blocks.
 static demag_status run_axes(demag_plan* P, ToepAxis* axes, int count, const char* what, cudaStream_t st,
-                             const float2* sympair = nullptr, const float* symreg = nullptr, int nsets = 2,
-                             int diag = 0) {
+                             const CompressedView* cv = nullptr, int diag = 0) {
   bool done[3] = {false, false, false};
   for (int i = 0; i < count; ++i) {
     if (done[i]) continue;
@@ -675,10 +685,11 @@ static demag_status run_axes(demag_plan* P, ToepAxis* axes, int count, const cha
     ToepLaunch a{};
     a.M = 0;
     a.pairstride = P->Lmax / 2;
-    a.sympair = sympair ? sympair : P->sympair;
-    a.symreg = symreg ? symreg : P->symreg;
+    a.sympair = cv ? cv->cpair : P->sympair;
+    a.symreg = cv ? cv->creg : P->symreg;
+    a.regstride = P->regstride;
     a.diag = diag;
-    a.nsets = nsets;
+    a.nsets = cv ? 3 : 2;
     int gx = 0;
     for (int j = i; j < count; ++j) {
       if (done[j] || ilog2i(P->L[axes[j].axis] / 2) != logn) continue;
@@ -839,7 +850,7 @@ extern "C" demag_status demag_apply_full_fibres(demag_plan* P, const float* m, f
   b.in_qstride = N;
   b.out = Y;
   b.out_bstride = 3 * N;
-  s = run_axes(P, &b, 1, "toeplitz_fft_kernel (fibres, axis 2)", st, nullptr, nullptr, 2, 1);
+  s = run_axes(P, &b, 1, "toeplitz_fft_kernel (fibres, axis 2)", st, nullptr, 1);
   if (s != DEMAG_OK) return s;
   // Z[k][q][i1][i2][i3]
   {
@@ -859,7 +870,7 @@ extern "C" demag_status demag_apply_full_fibres(demag_plan* P, const float* m, f
   c.in_qstride = N;
   c.out = Y;
   c.out_bstride = 3 * N;
-  s = run_axes(P, &c, 1, "toeplitz_fft_kernel (fibres, axis 3)", st, nullptr, nullptr, 2, 1);
+  s = run_axes(P, &c, 1, "toeplitz_fft_kernel (fibres, axis 3)", st, nullptr, 1);
   if (s != DEMAG_OK) return s;
   {
     const long tiles = (long)n2 * ((n1 + 31) / 32) * ((n3 + 31) / 32);
@@ -972,7 +983,7 @@ extern "C" demag_status demag_apply_tucker_compressed(demag_plan* P, int batch, 
     aoff += (long)r[p] * P->n[p];
     ooff += 3L * cv.rho[p] * r[p] * P->n[p];
   }
-  s = run_axes(P, ax, 3, "toeplitz_fft_kernel (compressed tucker)", st, cv.cpair, cv.creg, 3);
+  s = run_axes(P, ax, 3, "toeplitz_fft_kernel (compressed tucker)", st, &cv);
   if (s != DEMAG_OK || !out_core) return s;
   return launch_core_kron(P, batch, r, core, out_core, st);
 }
