@@ -216,8 +216,13 @@ void dispatch_symbol(demag_plan* P, int axis, int M, int nsets, const double* ge
 // 2048 356 against 418; at n = 4096 a column takes 512 threads, one block per SM, whose barriers nothing
 // covers: 873 against 796 us (922 with two threads per last step), so it ends at 2048.
 __host__ __device__ inline bool toep_in_registers(int N) { return N >= 256 && N <= 2048; }
-inline bool any_toep_in_registers(const demag_plan* P) {
-  return toep_in_registers(P->L[0] / 2) || toep_in_registers(P->L[1] / 2) || toep_in_registers(P->L[2] / 2);
+// Stride of a plan's table of their symbols: the longest such axis (0: none) and a place behind it, in
+// 128-byte rows (a warp loads 512 bytes at once).
+inline int toep_regstride(const demag_plan* P) {
+  int s = 0;
+  for (int L : P->L)
+    if (toep_in_registers(L / 2) && L + 32 > s) s = L + 32;
+  return s;
 }
 // Place of symbol value f < L in the order of that kernel's threads: thread f1 B + l (B = L / 256,
 // f = f1 + 16 f2) holds element s of its group's spectrum (rf_freq), four elements to a 16-byte load.

@@ -410,10 +410,9 @@ extern "C" demag_status demag_build_factors(const demag_grid_desc* d, demag_plan
       TRY_CUDA(cudaGetLastError());
     }
     const size_t pairs = (size_t)M * 6 * (P->Lmax / 2);
-    const bool regs = any_toep_in_registers(P);
-    P->regstride = regs ? P->Lmax + 32 : 0;  // 128-byte rows: a warp loads 512 bytes at once
+    P->regstride = toep_regstride(P);
     TRY_CUDA(cudaMalloc(&P->sympair, sizeof(float2) * pairs + sizeof(float) * (size_t)M * 6 * P->regstride));
-    if (regs) P->symreg = reinterpret_cast<float*>(P->sympair + pairs);
+    if (P->regstride) P->symreg = reinterpret_cast<float*>(P->sympair + pairs);
     for (int p = 0; p < 3; ++p) {
       const int N = P->L[p] / 2;
       const long total = (long)M * 2 * N;

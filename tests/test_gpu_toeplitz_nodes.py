@@ -57,3 +57,18 @@ def test_every_node_within_its_own_bound(n, R, kind):
                 ref = np.fft.irfft(np.fft.rfft(c) * X)[:, :n]
                 bound = 2.0 ** -24 * np.log2(L) * np.abs(t).sum() * np.linalg.norm(V[q][p], axis=1)
                 assert (np.linalg.norm(g[k, q] - ref, axis=1) <= bound).all(), (p, q, k)
+
+
+def test_symbols_of_a_short_axis_beside_a_long_one():
+    """The register kernel's table follows its own axes: 200 cells beside 4096 cost a few MB and not the
+    table of the long axis once more (25 MB at M = 128)."""
+    import paper_1212_3509_gb300 as D
+    used = []
+    for n1 in (100, 200, 100, 200):  # 100 cells have no such table; the first two load what is loaded once
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        P = D.demag_build_factors((n1, 4096, 1), (1 / 4096,) * 3, 257)
+        torch.cuda.synchronize()
+        used.append(free - torch.cuda.mem_get_info()[0])
+        P.close()
+    assert used[3] - used[2] < 8 << 20, used
