@@ -118,11 +118,15 @@ struct EnShared {
   EnGram<F> gram[3];
 };
 
+constexpr float kEnLarge = 1.3e36f;  // about 2^120: 32 of them stay finite
+
 // The three Grams g[0..2] (in shared memory) by the whole block.  The work is cut into items, 8 x 8
 // outputs over one segment of columns (at most 1024, so that the FP32 sums of a lane stay at 32
 // products), one warp each, 8 at a time: a lane takes every 32nd column of the segment, its 8 + 8
 // entries (read along the rows, coalesced) feed 64 products summed in registers, the lanes' sums are
-// added without loss (EnSum) by a transposing reduction, and segments in FP64 in a fixed order.
+// added without loss (EnSum) by a transposing reduction, and segments in FP64 in a fixed order.  Lane
+// sums beyond kEnLarge, infinite or not a number, whose two-sum would overflow or turn an infinity into
+// NaN, are added in FP64 instead.
 // Bound: the latency of an item's loads and reduction, so small ranks split the columns until every
 // warp has an item.  1024^3, ranks 8, R = 61 (270 blocks): 661 us when 64 x 64 tiles padded every
 // rank and each partial sum and derivative was formed in FP64; 35 us now.
@@ -190,17 +194,30 @@ __device__ void block_grams(const EnGram<F>* g, double* part) {
 #pragma unroll
           for (int c = 0; c < 8; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
       }
-      EnSum<F> v[64];
+      bool large = false;
+      if constexpr (std::is_same<F, float>::value) {
 #pragma unroll
-      for (int j = 0; j < 64; ++j) v[j].set(acc[j / 8][j % 8]);
-      en_halve<64>(v, 16);
-      en_halve<32>(v, 8);
-      en_halve<16>(v, 4);
-      en_halve<8>(v, 2);
-      en_halve<4>(v, 1);
-      // a lane is left with outputs 2 lane and 2 lane + 1
-      part[warp * 64 + 2 * lane] = v[0].value();
-      part[warp * 64 + 2 * lane + 1] = v[1].value();
+        for (int j = 0; j < 64; ++j) large = large || !(fabsf(acc[j / 8][j % 8]) <= kEnLarge);
+      }
+      if (__any_sync(0xffffffffu, large)) {
+#pragma unroll
+        for (int j = 0; j < 64; ++j) {
+          const double s = en_warp_sum((double)acc[j / 8][j % 8]);
+          if (lane == 0) part[warp * 64 + j] = s;
+        }
+      } else {
+        EnSum<F> v[64];
+#pragma unroll
+        for (int j = 0; j < 64; ++j) v[j].set(acc[j / 8][j % 8]);
+        en_halve<64>(v, 16);
+        en_halve<32>(v, 8);
+        en_halve<16>(v, 4);
+        en_halve<8>(v, 2);
+        en_halve<4>(v, 1);
+        // a lane is left with outputs 2 lane and 2 lane + 1
+        part[warp * 64 + 2 * lane] = v[0].value();
+        part[warp * 64 + 2 * lane + 1] = v[1].value();
+      }
     }
     __syncthreads();
     if (threadIdx.x < 64) {
