@@ -4,9 +4,11 @@
 // per node k and component q the three Toeplitz factors act along i1, i2, i3.
 // The modes are applied in the order 3, 2, 1.  Per node the nine products
 // share work (8 products of n^4 multiply-adds):
-//   axis 3:  Y_q = m_q x_3 S_k E (q = 1, 2),  Y_3 = m_3 x_3 S_k F,  S_k = c s omega_k
+//   axis 3:  Y_q = m_q x_3 E (q = 1, 2),  Y_3 = m_3 x_3 F
 //   axis 2:  U = Y_2 x_2 F + Y_3 x_2 E,  V = Y_1 x_2 E
-//   axis 1:  phi = sum_k (U_k x_1 E + V_k x_1 F)
+//   axis 1:  phi = sum_k (U_k x_1 S_k E + V_k x_1 S_k F),  S_k = c s omega_k
+// (S_k reaches 10^4 where E is small, so it goes with the last product: before it no field outgrows the
+// input's, E and F being integrals over a part of [-1, 1]).
 // and the node sum of the last stage is one contraction of length 2 n1 M.
 // Every field stays in the caller's layout [i3][i2][i1]: along axes 3 and 2
 // the rows of a product (everything but the contracted index) are contiguous
@@ -281,10 +283,19 @@ __global__ void __launch_bounds__(Cfg::NT, Cfg::OCC) mode_kernel(const __grid_co
     P2* a = As + buf * kBK * LDA;
 #pragma unroll
     for (int i = 0; i < LA; ++i) {
-      const T x = (T)ax[i], y = (T)ay[i];
+      const T x = (T)ax[i];
       P2 v;
-      v.x = ld_sw ? x - y : x + y;
-      v.y = ld_sw ? x + y : x - y;
+      if constexpr (KIND == 0 && std::is_same<T, float>::value) {
+        // half sums, which two values of any size have; the fields between the stages are half their
+        // values, and the axis-1 factors make up for it
+        const float y = 0.5f * ay[i], p = fmaf(0.5f, x, y), q = fmaf(0.5f, x, -y);
+        v.x = ld_sw ? q : p;
+        v.y = ld_sw ? p : q;
+      } else {
+        const T y = (T)ay[i];
+        v.x = ld_sw ? x - y : x + y;
+        v.y = ld_sw ? x + y : x - y;
+      }
       a[lk(i) * LDA + lr(i)] = v;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -396,7 +407,8 @@ __global__ void __launch_bounds__(Cfg::NT, Cfg::OCC) mode_kernel(const __grid_co
 //   skew ones x- -> even, x+ -> odd;
 //   non-uniform grid (two parts): the even / odd blocks of any matrix, part 0
 //   (x+ -> even, x- -> odd), part 1 (x- -> even, x+ -> odd).
-// Formed in FP64 and rounded once; the axis-3 factors carry c s omega_k.
+// Formed in FP64 and rounded once; the axis-1 factors carry c s omega_k, in FP32 twice that: the
+// axis-3 stage takes x+-/2, since the sum of two values of more than half the type's maximum overflows.
 
 struct ModeLayout {
   int h[3], ldh[3];
@@ -459,7 +471,7 @@ __global__ void factor_parts_kernel(int M, ModeLayout L, FactorSource s, T* out)
       v = 0.5 * (entry(a, j) + sj * entry(a, j2));
       if (s.fac) v = 0.5 * (v + (odd ? -0.5 : 0.5) * (entry(a2, j) + sj * entry(a2, j2)));
       if (j == j2) v *= 0.5;
-      if (p == 2) v *= s.scale[kt / 2];
+      if (p == 0) v *= (std::is_same<T, float>::value ? 2.0 : 1.0) * s.scale[kt / 2];
     }
     out[idx] = (T)v;
   }
