@@ -503,13 +503,13 @@ demag_status demag_set_wait_limit(demag_plan* plan, double seconds);
  * (demag_stray_field_exact) follow this call too.  Both give the same values
  * to rounding (the same
  * products, accumulated in another order); other grids and forms always run
- * the chain.  Without this call the forward application takes the autotuner's
- * choice (demag_autotune, kind 9), else the fused schedule where ext1^2 ext2,
- * the extents of the folded layout, is at least 4.5e6 (a cube of about 165^3;
- * with fewer than 8 nodes, where the grid has 2^20 cells in that layout) and
- * the chain elsewhere; the adjoint and the stray field take the fused one
- * where ext1^2 ext2 is at least 1.2e7 (about 229^3).  Build-only; no
- * counterpart in the paper. */
+ * the chain.  Without this call all three take the autotuner's choice
+ * (demag_autotune, kind 9); without that too, the forward application takes
+ * the fused schedule where ext1^2 ext2, the extents of the folded layout, is
+ * at least 4.5e6 (a cube of about 165^3; with fewer than 8 nodes, where the
+ * grid has 2^20 cells in that layout) and the chain elsewhere, the adjoint and
+ * the stray field the fused one where ext1^2 ext2 is at least 1.2e7 (about
+ * 229^3).  Build-only; no counterpart in the paper. */
 demag_status demag_set_fused(demag_plan* plan, int enable);
 
 /* The forward schedule a plan's next full-format application in `prec`
@@ -576,8 +576,9 @@ demag_status demag_profile_launch(demag_plan* plan, long long i, int* family, do
 
 /* demag_autotune(plan, 1) turns tuning on for this plan: from then on
  *  - the first Toeplitz-FFT launch of each shape (FFT length, number of column
- *    blocks, M) times every node-group size M, M/2, ..., 1 (one warm-up and
- *    three timed launches each, on the call's stream, which is synchronised)
+ *    blocks, M) times every node-group size M, M/2, ..., 1 (rounded up to even
+ *    numbers and down to 2 where two nodes share a transform, on axes of 129
+ *    to 2048 cells; one warm-up and three timed launches each, on the call's stream, which is synchronised)
  *    and keeps the fastest for later launches of that shape;
  *  - tensor-core state created afterwards (first DEMAG_TF32X3 / DEMAG_BF16X3
  *    use) times, per mode-product stage program, one knob after the other
@@ -588,7 +589,8 @@ demag_status demag_profile_launch(demag_plan* plan, long long i, int* family, do
  *    in one outer index, the store boxes {per epilogue warp, one 128-row box
  *    per chunk} (operands as they are, stage timed alone); then, where the
  *    grid has the fused BF16x3 forward schedule (demag_set_fused), that
- *    schedule's two launches against the three-stage chain.
+ *    schedule's two launches against the three-stage chain; the adjoint and
+ *    the analytic stray field follow that choice.
  * No knob changes the arithmetic of an output element: tuned and untuned
  * results agree bit for bit.  The tuning launches write the call's own
  * outputs.  No tuning happens while the stream is being captured.

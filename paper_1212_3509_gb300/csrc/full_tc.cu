@@ -2017,7 +2017,7 @@ struct TcState {
   bool fused;
   int sched;              // forward schedule (1 fused, 0 chain): the tuner's choice, else sched0
   int sched0;             // untuned forward schedule, by size
-  int sched_adj;          // schedule of the adjoint and the analytic stray field, by size
+  int sched_adj;          // schedule of the adjoint and the analytic stray field: the tuner's choice, else by size
   S12Launch s12;
   S12Launch s12a;         // the adjoint's fused launch (Z with 3M fields)
   // analytic stray field: the forward stage programs with the derivative
@@ -2471,14 +2471,15 @@ static demag_status set_knob(demag_plan* P, TcState* S, int prog, int knob, int 
   return DEMAG_OK;
 }
 
-// Tuned entry kind of the forward schedule (BF16x3): 1 fused, 0 chain; key (0, 1, 0).
+// Tuned entry kind of the schedule (BF16x3): 1 fused, 0 chain; key (0, 1, 0).  Timed on the forward
+// application; the adjoint and the stray field follow it.
 constexpr int kTuneSchedule = 9;
 
 // Apply tuned entries already in the plan (a loaded cache) to its programs.
 static demag_status apply_tuned(demag_plan* P, TcState* S) {
   if (S->fused)
     for (const demag_plan::Tuned& t : P->tuned)
-      if (t.kind == kTuneSchedule && (t.value == 0 || t.value == 1)) S->sched = t.value;
+      if (t.kind == kTuneSchedule && (t.value == 0 || t.value == 1)) S->sched = S->sched_adj = t.value;
   for (int prog = 0; prog < kPrograms; ++prog) {
     if (S->small[prog] || (prog >= kChain && !S->fused)) continue;
     for (int knob = 0; knob < 4; ++knob) {
@@ -2604,7 +2605,7 @@ static demag_status tune_programs(demag_plan* P, TcState* S, cudaStream_t st) {
     s = time_sched(1, &mf);
     if (s == DEMAG_OK) s = time_sched(0, &mc);
     if (s == DEMAG_OK) {
-      S->sched = mc < mf ? 0 : 1;
+      S->sched = S->sched_adj = mc < mf ? 0 : 1;
       demag_plan::Tuned t;
       t.kind = kTuneSchedule;
       t.key[0] = 0;
