@@ -506,8 +506,8 @@ demag_status demag_set_wait_limit(demag_plan* plan, double seconds);
  * the chain.  Without this call all three take the autotuner's choice
  * (demag_autotune, kind 9); without that too, the forward application takes
  * the fused schedule where ext1^2 ext2, the extents of the folded layout, is
- * at least 4.5e6 (a cube of about 165^3; with fewer than 8 nodes, where the
- * grid has 2^20 cells in that layout) and the chain elsewhere, the adjoint and
+ * at least 4.5e6 (a cube of about 165^3; with fewer than 8 nodes 1.5e6 and
+ * 2^20 cells in that layout) and the chain elsewhere, the adjoint and
  * the stray field the fused one where ext1^2 ext2 is at least 1.2e7 (about
  * 229^3).  Build-only; no counterpart in the paper. */
 demag_status demag_set_fused(demag_plan* plan, int enable);

@@ -2754,13 +2754,16 @@ demag_status tc_prepare(demag_plan* P, demag_precision prec, cudaStream_t st) {
     // ext1^2 ext2.  BF16x3, R = 41, chain against fused, us: 128^3 385 / 418, 160^3 760 / 819,
     // 176^3 1214 / 1154, 256^3 2761 / 2108, 53 x 204 x 181 692 / 1040, 256 x 128 x 128 697 / 606,
     // 128 x 256 x 256 1447 / 1588 (41 grids, each also at R = 11, 21, 61: the same side but for ties).
-    // With fewer than 8 nodes the two differ by 10 us or so on the grids between; those keep the
-    // line at 2^20 split cells.
-    S->sched0 = x1 * x1 * x2 >= 4500000LL || (M < 8 && x1 * x2 * x3 >= (1LL << 20)) ? 1 : 0;
+    // With fewer than 8 nodes, where fixed costs weigh more, the two are close from 1.5e6 on: those grids
+    // keep the older line of 2^20 split cells (M = 5: 128 x 96 x 96 107 / 119, 160 x 96 x 80 121 / 120, 144^3
+    // 269 / 268, 160^3 263 / 278), and below it the chain is the faster by far (96 x 128 x 128 135 / 155,
+    // 64 x 192 x 192 212 / 267, 53 x 204 x 181 278 / 369).
+    const long long x112 = x1 * x1 * x2;
+    S->sched0 = x112 >= 4500000LL || (M < 8 && x112 >= 1500000LL && x1 * x2 * x3 >= (1LL << 20)) ? 1 : 0;
     // The adjoint (three targets per unit instead of two, mode-1 tiles formed twice) and the stray
     // field (one fused launch per direction where the chain shares stages): 192^3 1192 / 1200 and
     // 3064 / 3043, 224^3 2171 / 2198, 240 x 208 x 66 1042 / 981, 256^3 2751 / 2569 and 7046 / 6189.
-    S->sched_adj = x1 * x1 * x2 >= 12000000LL ? 1 : 0;
+    S->sched_adj = x112 >= 12000000LL ? 1 : 0;
     S->sched = S->sched0;
     if (S->fused) {
       S12Launch& Z = S->s12;

@@ -63,3 +63,19 @@ def test_every_direction_follows_the_tuned_choice(D, fused, tmp_path):
     assert D.demag_autotune_load(P, str(path)) == len(lines)
     assert _launches(D, P) == (FUSED if fused else CHAIN)
     P.close()
+
+
+# forward line 4.5e6 of ext1^2 ext2 (with fewer than 8 nodes 1.5e6 and 2^20 cells), the others' 1.2e7; grids
+# whose number of cells says otherwise among them
+@pytest.mark.parametrize("n,R,forward,others", [
+    ((160, 160, 17), 41, 0, 0), ((128, 96, 96), 41, 0, 0), ((53, 204, 181), 41, 0, 0),  # 4.1e6, 1.6e6, 0.9e6
+    ((176, 160, 20), 41, 1, 0), ((240, 208, 20), 17, 1, 0),                             # 5.0e6, 11.98e6
+    ((240, 224, 20), 17, 1, 1), ((256, 256, 17), 5, 1, 1),                              # 12.9e6, 16.8e6
+    ((128, 96, 96), 15, 1, 0), ((128, 96, 96), 17, 0, 0), ((128, 96, 64), 15, 0, 0),    # 7 and 8 nodes; few cells
+    ((53, 204, 181), 11, 0, 0), ((96, 128, 128), 11, 0, 0)])                            # many cells, short first axis
+def test_untuned_choice_by_size(D, n, R, forward, others):
+    P = D.demag_build_factors(n, (1 / max(n),) * 3, R)
+    got = _launches(D, P)
+    assert D.demag_forward_schedule(P, "bf16x3") == forward
+    P.close()
+    assert got == ((FUSED if forward else CHAIN)[0],) + (FUSED if others else CHAIN)[1:]
