@@ -3161,6 +3161,8 @@ demag_status tc_batch_create(demag_plan* const* plans, int count, demag_precisio
       ++SB.count;
     }
   }
+  // the groups that become segments: slot 0 of a fused grid, all slots of a chain grid but a thin last stage
+  auto used = [&](int i, int st3) { return B->fused[order[i]] ? st3 == 0 : !(st3 == 2 && thin3[i]); };
   // Tiles wider than 128 columns (an axis half above 128: long films, non-uniform grids) would hold
   // the whole launch to one CTA per SM (launch_segs).  Where they carry less than half of its output
   // they are cut into equal ones of at most 128: 16 uneven grids with two 512 x 512 x 4 films 7.20 ms
@@ -3168,16 +3170,19 @@ demag_status tc_batch_create(demag_plan* const* plans, int count, demag_precisio
   // 453 us, 256^3 non-uniform 3.28 against 3.97 ms), which keep their A operand's rows longer.
   {
     double wide = 0, all = 0;
-    for (const TcGroup& gg : g) {
-      const double w = (double)gg.njobs * gg.rows * gg.n_a;
-      all += w;
-      if (gg.bn > 128) wide += w;
-    }
+    for (int i = 0; i < count; ++i)
+      for (int st3 = 0; st3 < 3; ++st3) {
+        if (!used(i, st3)) continue;
+        const TcGroup& gg = g[st3 * count + i];
+        const double w = (double)gg.njobs * gg.rows * gg.n_a;
+        all += w;
+        if (gg.bn > 128) wide += w;
+      }
     if (wide > 0 && wide < 0.5 * all)
       for (int i = 0; i < count; ++i)
         for (int st3 = 0; st3 < 3; ++st3) {
           TcGroup& G = g[st3 * count + i];
-          if (G.bn <= 128) continue;
+          if (G.bn <= 128 || !used(i, st3)) continue;
           const TcState* S = state(plans[order[i]], prec);
           const int axis = B->fused[order[i]] && st3 == 0 ? 2 : st3;
           const int tiles = (G.n_a + 127) / 128;
@@ -3199,7 +3204,7 @@ demag_status tc_batch_create(demag_plan* const* plans, int count, demag_precisio
       const bool fz = B->fused[order[i]] != 0;
       if (fz != (pass == 1)) continue;
       const int st3 = pass == 0 ? 0 : pass - 1;
-      if (st3 == 2 && thin3[i]) continue;  // in the CUDA-core launch after this one
+      if (!used(i, fz ? 0 : st3)) continue;  // a thin last stage: in the CUDA-core launch after this one
       const int gi = fz ? i : st3 * count + i;
       if (g[gi].ntiles <= 0) continue;
       TcSeg q = whole_seg(g[gi], gi, acc);
@@ -3210,9 +3215,9 @@ demag_status tc_batch_create(demag_plan* const* plans, int count, demag_precisio
       if (!fz && st3 < 2) q.done = 2 * i + st3;
       segs.push_back(q);
       acc += g[gi].ntiles;
+      B->maxbn = std::max(B->maxbn, g[gi].bn);
     }
   }
-  for (const TcGroup& gg : g) B->maxbn = std::max(B->maxbn, gg.bn);
   B->nsegs = (int)segs.size();
   B->total = acc;
   B->nctr = 2 * count;

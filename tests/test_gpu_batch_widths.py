@@ -86,3 +86,24 @@ def test_cached_width_that_splits_a_store_box_is_not_taken(D, tmp_path):
         D.demag_apply_full(P, m, b, "bf16x3")
         assert torch.equal(a, b)
     P.close()
+
+
+@pytest.mark.parametrize("shapes", [[((256, 256, 300), True), ((300, 300, 12), False), ((64, 64, 64), False)],
+                                    [((256, 256, 40), True), ((300, 20, 18), False)],
+                                    [((512, 512, 4), False), ((128, 64, 64), True)]])
+def test_batch_of_fused_grids_films_and_chains(D, shapes):
+    """Only the groups that run decide how wide tiles are taken: the mode-3 stage of a fused grid, not its
+    unused chain stages; the stages of a film without its last one."""
+    plans = [_plan(D, n, True, 11) for n, _ in shapes]
+    ms = [dev(synth.random_unit_m(n, 70 + i)) for i, (n, _) in enumerate(shapes)]
+    single = [torch.empty(n[2], n[1], n[0], device="cuda") for n, _ in shapes]
+    for P, (_, fused), m, o in zip(plans, shapes, ms, single):
+        D.demag_set_fused(P, fused)
+        D.demag_apply_full(P, m, o, "bf16x3")
+    out = [torch.full_like(o, float("nan")) for o in single]
+    D.demag_apply_full_batched(plans, ms, out, "bf16x3")
+    for a, b in zip(out, single):
+        assert torch.equal(a, b)
+    for P in plans:
+        D.demag_sync_status(P)
+        P.close()
