@@ -509,10 +509,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const __grid_con
         epi_signal(L.counters, pend, pend_n, pend_tma, 0, lane);
         pend = -1;
       }
-      // (a zero limit is taken at its word here, once per tile: the try of a bounded wait alone may
-      // block for longer than a short tile takes)
-      if (L.wait_ns == 0 ? !ptx::mbar_test_wait(&tfull[buf], tph)
-                         : !ptx::mbar_wait(&tfull[buf], tph, abort, L.wait_ns)) {
+      if (!ptx::mbar_wait(&tfull[buf], tph, abort, L.wait_ns)) {
         tc_fail(abort, L.status);
         break;
       }

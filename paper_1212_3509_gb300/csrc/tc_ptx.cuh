@@ -68,29 +68,19 @@ __device__ __forceinline__ bool mbar_try_wait_suspend(uint64_t* bar, uint32_t pa
   return ok != 0;
 }
 
-// The test alone, never blocking (try_wait may suspend the thread for some microseconds).
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 // Wait for the phase with the given parity to complete.  Gives up after
 // `limit_ns` nanoseconds or when *abort becomes non-zero; returns success.
+// No try blocks for longer than the limit, so that a very short one (zero,
+// say) runs out on a phase that is not complete yet.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
+  const uint32_t ns = limit_ns < 10000 ? (uint32_t)limit_ns : 10000u;
+  if (mbar_try_wait_suspend(bar, parity, ns)) return true;
   const uint64_t t0 = globaltimer();
   for (;;) {
-    if (mbar_try_wait_suspend(bar, parity, 10000)) return true;
     if (*abort) return false;
-    if (globaltimer() - t0 > limit_ns) return false;
+    if (globaltimer() - t0 >= limit_ns) return false;
+    if (mbar_try_wait_suspend(bar, parity, ns)) return true;
   }
 }
 
