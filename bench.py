@@ -10,7 +10,9 @@ R = 61), where one application produces the CP output of rank 30*3*4.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Prints ONE JSON line on rank 0.  Under torchrun (N > 1) every rank runs the
+Prints ONE JSON line on rank 0: the headline in full and the figures of every
+other row; the complete record of all rows goes to standard error as one JSON
+line.  Under torchrun (N > 1) every rank runs the
 same workload independently (the operator does not shard across GPUs here:
 replicas only) and `value` is the total over ranks divided by the slowest
 rank's time.  `--impl reference` times the FP64 CPU oracle on bounded samples
@@ -72,6 +74,34 @@ def ncu_traffic(kernel, units, unit_key):
 
 # FP32 CUDA-core peak of a GB300: 152 SMs x 128 FP32 lanes x 2 flops (FMA) x 2.07 GHz
 FP32_SIMT_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
+
+
+# keys of the result line that are printed as they are; the other rows as their figures (SHORT_KEYS)
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "roofline", "e2e", "gpu_launches", "clocks", "cpu_baseline",
+             "rel_l2_full")
+SHORT_KEYS = ("value", "apps_per_s", "rel_l2", "rel_l2_sampled_max", "frac")
+
+
+def short(v):
+    """The figures of a row: its SHORT_KEYS and those of the rows inside it, to six digits."""
+    out = {}
+    for k, x in v.items():
+        if isinstance(x, dict):
+            if s := short(x):
+                out[k] = s
+        elif k in SHORT_KEYS and isinstance(x, (int, float)):
+            out[k] = float(f"{x:.6g}")
+    return out
+
+
+def line_of(result):
+    """The one line that is printed: readers keep a few KB of it, and the full record (autotuner entries,
+    the energy study's tables, notes) is 20 KB, which goes to standard error."""
+    line = {k: result[k] for k in LINE_KEYS if k in result}
+    rows = {k: short(v) for k, v in result.items() if k not in line and isinstance(v, dict)}
+    line.update({k: v for k, v in rows.items() if v})
+    return line
 
 
 def parse():
@@ -355,7 +385,7 @@ def run_ours(args, world, rank, local):
     else:
         tpeak = FP32_SIMT_PEAK_TFLOPS
         tpeak_note = "FP32 FMA peak from unit counts and max clock (152 SMs x 128 lanes x 2 x 2.07 GHz)"
-        roofline = {"kernel": "gemm_tn_kernel (CUDA-core mode products), all stages of one application",
+        roofline = {"kernel": "mode_kernel (CUDA-core mode products), all stages of one application",
                     "bound": "alu", "achieved": achieved_tflops, "peak": tpeak, "unit": "TFLOP/s",
                     "frac": achieved_tflops / tpeak, "traffic": None, "peak_source": tpeak_note,
                     "algorithmic_flops_per_app": flops_app, "launches_per_app": gemm_n / args.steps,
@@ -673,7 +703,8 @@ def run_ours(args, world, rank, local):
         for k in [k for k in batch if k.startswith("_")]:
             del batch[k]
         result["uneven_batch"] = batch
-    print(json.dumps(result), flush=True)
+    print(json.dumps({"details": result}), file=sys.stderr, flush=True)
+    print(json.dumps(line_of(result)), flush=True)
 
 
 def run_c2_128(args, D, stream):
