@@ -27,7 +27,8 @@
  *    the footnote to Cor. 3); a magnetization is float [3][n3][n2][n1].
  *  - Memory: every data pointer is a DEVICE pointer owned by the caller; the
  *    library never frees or retains it after the call returns.  The plan owns
- *    its generators, symbols, dense factor matrices and workspace.
+ *    its generators, symbols, factor matrices and workspace, and a memory pool
+ *    for the scratch of the structured energies, which keeps up to 64 MiB.
  *  - Streams: `stream` is a cudaStream_t (NULL = legacy default stream).  All
  *    compute entry points are asynchronous on that stream, except the
  *    host-driven ones documented as synchronous (kernel compression,
@@ -154,7 +155,10 @@ size_t demag_symbols_size(const demag_plan* plan);
  * (mode 1: F m1, E m2, E m3; mode 2: E Y1 + F Y2, E Y3; mode 3 with the node
  * sum folded into the contraction).  The first call of a precision allocates
  * its workspace (so make it before any stream capture).  m and phi must not
- * overlap. */
+ * overlap.  Finite values of any size are taken in DEMAG_FP32 and DEMAG_FP64;
+ * an infinity or NaN in m leaves infinities and NaNs in phi, and which of the
+ * two stands where is not specified (each form works on sums and differences
+ * of mirror cells). */
 demag_status demag_apply_full(demag_plan* plan, const float* m, float* phi,
                               demag_precision prec, void* stream);
 
@@ -247,7 +251,10 @@ demag_status demag_graph_launch(demag_graph* graph, void* stream);
 int demag_graph_kernel_count(const demag_graph* graph);
 void demag_graph_destroy(demag_graph* graph);
 
-/* Allocate the full-format workspace of `prec` now (idempotent). */
+/* Allocate the full-format workspace of `prec` now (idempotent).  DEMAG_FP32
+ * and DEMAG_FP64: 3 (M + min(M, max(1, c))) fields of 4 or 8 bytes an entry, c
+ * the number of nodes whose three fields fit into 256 MiB (on small grids
+ * all nodes go through a mode in one launch). */
 demag_status demag_reserve_workspace(demag_plan* plan, demag_precision prec);
 
 /* Adjoint: g^(q) = (P^(q))^T y for q = 1..3.  E is even and F odd in d (Sec.
@@ -528,7 +535,7 @@ int demag_forward_schedule(const demag_plan* plan, demag_precision prec);
  * GPU (an allocation from a library would fail or fragment it), loops where
  * an allocation would implicitly synchronise the device, and hosts whose
  * plugin rules forbid allocation.  No plan is needed and nothing is
- * allocated: the nodes, generators, dense factors and intermediate fields
+ * allocated: the nodes, generators, factors and intermediate fields
  * live in one fixed device array of 32 MiB inside the library, which every
  * GPU that loads the library keeps until the process exits.
  * desc: the grid, as for demag_build_factors; m: float [3][n3][n2][n1] and

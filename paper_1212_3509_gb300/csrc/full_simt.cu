@@ -615,7 +615,8 @@ static cudaError_t launch_mode_cfg(demag_plan* P, ModeStage S, int split, cudaSt
 // and the exchange of a split sum), over the configuration's rate, which falls
 // when fewer blocks are resident than fit.  The rates and overheads were fitted
 // to the times of every configuration at 13 grids from 16^3 to 192^3 (R = 41):
-// the choice is within 2% of the fastest on average.  E.g. axis 3 of 128^3:
+// for the stages of axes 3 and 2 the choice is within 2% of the fastest on
+// average (the split sum of axis 1 needs the terms below).  E.g. axis 3 of 128^3:
 // 128 x 64 tiles 398 us, 256 x 32 413, 128 x 32 447, 256 x 16 493, 64 x 16 705;
 // of 16^3: 10.2, 10.2, 11.0, 10.1, 7.0; axis 1 (the node sum) of 48^3: 128 x 64
 // 129, split over 4 blocks 45, 64 x 16 over 8 blocks 26.5.
@@ -624,7 +625,6 @@ struct ModeShape {
   double rate, fill;  // at full occupancy; exponent of the resident share below it
 };
 
-//
 // A split sum runs as clusters, and three things decide its time beside that:
 // the longest node range (20 nodes over 6 or 7 blocks: 4 and 3); the share of the
 // block slots that clusters of one size can fill (as
@@ -1062,7 +1062,7 @@ extern "C" int demag_graph_kernel_count(const demag_graph* g) { return g ? g->ke
 // from a library would fail or fragment it), latency-critical loops where
 // an allocation would implicitly synchronise the device, and embedders whose
 // plugin rules forbid allocation.  Everything this call needs beyond the
-// caller's input and output (nodes, generators, dense factors and the
+// caller's input and output (nodes, generators, factor parts and the
 // intermediates of the mode-product chain) lives in one file-scope device
 // array of fixed size, which every GPU that loads the library keeps until
 // the process exits.  The arithmetic is that of demag_apply_full with
@@ -1143,7 +1143,8 @@ extern "C" demag_status demag_apply_full_noalloc(const demag_grid_desc* d, const
   const size_t N = (size_t)P.n[0] * P.n[1] * P.n[2];
 
   // scratch layout: nodes [3][M], scale [M], generators [M][2][3][glen] (FP64),
-  // dense factors [M][2][sum n_p^2] and the chain's fields Y (3) + U, V (2M) (FP32)
+  // factor parts and the chain's fields Y (3) + U, V (2M) (FP32); the limit counts [M][2][sum n_p^2] entries
+  // for the factors, about twice what their parts take
   const size_t b_nodes = na_align(sizeof(double) * 3 * M);
   const size_t b_scale = na_align(sizeof(double) * M);
   const size_t b_gen = na_align(sizeof(double) * (size_t)M * 6 * P.glen);
