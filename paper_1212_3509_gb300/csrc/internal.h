@@ -55,14 +55,14 @@ struct demag_plan {
   double* scale = nullptr;   // [M]: c * s * omega_k
   double* gend = nullptr;    // [M][2][3][glen]: derivative generators dE/s, dF/s (lazily, analytic stray field)
 
-  // dense factor matrices of the full path, per precision (device, lazily built)
-  // layout [M][2][3] blocks of n_p x n_p (row-major T[i][j] = gen[i-j]),
-  // axis-3 blocks carry the scale c*s*omega_k.
+  // factors of the full path on CUDA cores, per precision (device, lazily built):
+  // per node, type and axis the parts that map half sums to output halves
+  // (full_simt.cu, factor_parts_kernel); those of axis 1 carry the scale c*s*omega_k.
   float* T32 = nullptr;
   double* T64 = nullptr;
   // non-uniform tensor grid (demag_build_factors_nonuniform): the factors are
-  // dense, not Toeplitz.  fac64 holds them in FP64 in the T64 layout without
-  // the scale; gen64, sym and the twiddles stay unset (no FFT forms).
+  // dense, not Toeplitz.  fac64 holds them in FP64 without the scale, layout
+  // [M][2][3] blocks of n_p x n_p, row-major; gen64, sym and the twiddles stay unset (no FFT forms).
   bool nonuniform = false;
   double* fac64 = nullptr;   // [M][2][tgroup]
   float* T32t = nullptr;     // transposed tables for the adjoint (CUDA cores)

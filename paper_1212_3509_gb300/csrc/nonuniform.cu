@@ -7,8 +7,8 @@
 //   F[i][j] = int_{I_j} (xi_i - y) exp(-tau^2 (xi_i - y)^2) dy = int_a^b x exp(-tau^2 x^2) dx,
 // a = xi_i - y_{j+1} < b = xi_i - y_j, in coordinates scaled by the longest
 // domain edge s.  They are no longer Toeplitz (the cell widths differ), so the
-// plan keeps them as full matrices in the layout of the dense factor tables;
-// the full-format chains then run unchanged.
+// plan keeps them as full matrices, from which the full-format chains take
+// their factors.
 #include <cmath>
 
 #include "internal.h"

@@ -605,14 +605,15 @@ static cudaError_t launch_logn(demag_plan* P, int logn, const ToepLaunch& a, int
 
 // Nodes per block (an even number, or all, in the register kernel).  Each
 // block transforms its columns once and reuses the spectra for kgroup nodes,
-// so large groups save forward FFTs, while small groups give more blocks.  Default: the largest group that still yields
-// eight blocks per SM; in the register kernel, where a forward transform costs
-// as much as two nodes, half of the blocks that are resident at once (CP 2048,
-// r = 4, 8 items 105 -> 55 us, TT 700, ranks 3 5, 3 items 30 -> 20 us; all of
-// the resident ones 62 and 22 us, and CP 400, 4 items 14 against 17 us); with
-// autotuning on, the candidates M, M/2, M/4, ..., 1 (rounded up to even numbers
-// and down to 2 in the register kernel) are timed once per (FFT length, column
-// blocks, M) and the fastest is kept.
+// so large groups save forward FFTs, while small groups give more blocks.
+// Default: the largest group that still yields eight blocks per SM; in the
+// register kernel, where a forward transform costs as much as two nodes, half
+// of the blocks that are resident at once (CP 2048, r = 4, 8 items 105 -> 55
+// us, TT 700, ranks 3 5, 3 items 30 -> 20 us; all of the resident ones 62 and
+// 22 us, and CP 400, 4 items 14 against 17 us); with autotuning on, the
+// candidates M, M/2, M/4, ..., 1 (rounded up to even numbers and down to 2 in
+// the register kernel) are timed once per (FFT length, column blocks, M) and
+// the fastest is kept.
 static cudaError_t pick_kgroup(demag_plan* P, int logn, ToepLaunch& a, int gx, cudaStream_t st) {
   const int M = a.M;
   // nodes go in pairs in the register kernel: groups of an even number, or all nodes, so that the
