@@ -570,11 +570,12 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p5_kernel(const __grid_
 // shared memory once per transform, and a product with the kernel or the
 // Hermitian extension takes the spectrum in the lanes' frequency order.  With
 // every radix-16 pass (and the staging before it) through shared memory, P3 of
-// 256^3 had its wavefronts 71% and its issue slots 62% busy; it now runs half
-// the wavefronts and waits for HBM.  Before / now, us per pass: 256^3 potential
-// P1 158 / 129, P2 299 / 223 (5.4 TB/s), P3 518 / 448, P4 94 / 82, P5 61 / 47;
-// field P3 of 150 x 100 x 60 (length 128, whose fibres also collided in the
-// banks) 176 / 119.  Registers: 64 at 512 threads (lengths of 512) and 80 at 256
+// 128 x 256 x 256 had its wavefronts 70% and its issue slots 61% busy; it now
+// runs 36% fewer wavefronts of shared memory (22% fewer in all; 63% busy, issue
+// 57%, HBM 34%) and waits for its loads and for shared memory at 16 warps per SM
+// (264 -> 229 us).  Before / now, us per pass: 256^3 potential P1 158 / 128, P2
+// 299 / 225 (5.4 TB/s), P3 518 / 450, P4 94 / 82, P5 61 / 48; field P3 of 150 x
+// 100 x 60 (length 128, whose fibres also collided in the banks) 176 / 119.  Registers: 64 at 512 threads (lengths of 512) and 80 at 256
 // keep 32 and 24 warps per SM; P3 takes 128.
 constexpr bool rf_length(int N) { return N >= 32 && N <= 512; }
 template <int LOGN> struct R3 {

@@ -212,8 +212,8 @@ __global__ void generators_kernel(int M, int glen, GridInfo g, const double* nod
 demag_status require_uniform(demag_plan* plan, const char* what);
 void dispatch_symbol(demag_plan* P, int axis, int M, int nsets, const double* gen, float* sym, cudaStream_t st);
 // Axes whose circulant transform the structured kernel keeps in registers: L = 2N of 512 to 4096 points.
-// Against in-place passes (CP, r = 4, 64 items, GB300): n = 200 33 against 70 us, 1024 150 against 241,
-// 2048 356 against 418; at n = 4096 a column takes 512 threads, one block per SM, whose barriers nothing
+// Against in-place passes (CP, r = 4, R = 61, 64 items, GB300, graph replays): n = 129 38 against 92 us,
+// 400 73 against 154, 1024 148 against 237, 2048 353 against 415; at n = 4096 a column takes 512 threads, one block per SM, whose barriers nothing
 // covers: 873 against 796 us (922 with two threads per last step), so it ends at 2048.
 __host__ __device__ inline bool toep_in_registers(int N) { return N >= 256 && N <= 2048; }
 // Stride of a plan's table of their symbols: the longest such axis (0: none) and a place behind it, in

@@ -365,15 +365,15 @@ __global__ void __launch_bounds__(256, ToepCfg<LOGN>::minblocks)
 // buffer serve the inner exchange before they take its results, and two
 // buffers alternate, so a pair of nodes costs one block barrier.
 //
-// Bound by the wavefronts of shared memory and L1 (76% busy; issue 64%, FP32 pipe
+// Bound by the wavefronts of shared memory and L1 (74% busy; issue 62%, FP32 pipe
 // 59%) at 16 warps per SM, held there by 128 registers (X, the values and two
-// sets of 8 twiddles): per 16 points and pair
-// of nodes 32 wavefronts of symbols and 128 of the two exchanges, where the
-// in-place passes take about 240 per node, four block barriers against one.
-// GB300, R = 61: TT 1024 cells, ranks 8 8, 16 items 338 -> 238 us; CP 1024,
-// r = 4, 64 items 241 -> 152 us; a column's error 2.1e-7 -> 1.3e-7.  Five blocks
-// of 128 threads per SM (96 registers, spills) 284 us; the next symbols
-// prefetched into L1 156 instead of 150 us for that CP batch.
+// sets of 8 twiddles): per 16 points and pair of nodes 32 wavefronts of symbols
+// and 128 of the two exchanges, where the in-place passes take about 240 per
+// node, four block barriers against one.  GB300, R = 61: TT 1024 cells, ranks 8
+// 8, 16 items 338 -> 238 us; CP 1024, r = 4, 64 items 241 -> 152 us; a column's
+// error 2.1e-7 -> 1.3e-7.  Five blocks of 128 threads per SM (96 registers,
+// spills) 284 us for the trains; the next symbols prefetched into L1 156
+// instead of 150 us for the CP batch.
 template <int LOGN> struct RegToep {
   static constexpr int L = 2 << LOGN;
   static constexpr int B = L / 256;
