@@ -129,7 +129,7 @@ constexpr float kEnLarge = 1.3e36f;  // about 2^120: 32 of them stay finite
 // NaN, are added in FP64 instead.
 // Bound: the latency of an item's loads and reduction, so small ranks split the columns until every
 // warp has an item.  1024^3, ranks 8, R = 61 (270 blocks): 661 us when 64 x 64 tiles padded every
-// rank and each partial sum and derivative was formed in FP64; 35 us now.
+// rank and each partial sum and derivative was formed in FP64; 33 us now.
 template <typename F>
 __device__ void block_grams(const EnGram<F>* g, double* part) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

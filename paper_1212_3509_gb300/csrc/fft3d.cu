@@ -575,8 +575,9 @@ __global__ void __launch_bounds__(F3<LOGN>::BLOCK) fft3d_p5_kernel(const __grid_
 // 57%, HBM 34%) and waits for its loads and for shared memory at 16 warps per SM
 // (264 -> 229 us).  Before / now, us per pass: 256^3 potential P1 158 / 128, P2
 // 299 / 225 (5.4 TB/s), P3 518 / 450, P4 94 / 82, P5 61 / 48; field P3 of 150 x
-// 100 x 60 (length 128, whose fibres also collided in the banks) 176 / 119.  Registers: 64 at 512 threads (lengths of 512) and 80 at 256
-// keep 32 and 24 warps per SM; P3 takes 128.
+// 100 x 60 (length 128, whose fibres also collided in the banks) 176 / 119.
+// Registers: 64 at 512 threads (lengths of 512) and 80 at 256 keep 32 and 24
+// warps per SM; P3 takes 128.
 constexpr bool rf_length(int N) { return N >= 32 && N <= 512; }
 template <int LOGN> struct R3 {
   static constexpr bool OK = rf_length(1 << LOGN);
